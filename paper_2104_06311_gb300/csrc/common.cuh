@@ -26,9 +26,8 @@ __device__ __forceinline__ float qam_level(float x) {
   if (MB == 2) {
     return x >= 0.f ? 0.70710678118654752f : -0.70710678118654752f;
   } else {
-    const float s = x * 3.16227766016837933f;
-    float l = s >= 0.f ? (s > 2.f ? 3.f : 1.f) : (s < -2.f ? -3.f : -1.f);
-    return l * 0.31622776601683793f;
+    const float l = fabsf(x * 3.16227766016837933f) > 2.f ? 3.f * 0.31622776601683793f : 0.31622776601683793f;
+    return x >= 0.f ? l : -l;
   }
 }
 
