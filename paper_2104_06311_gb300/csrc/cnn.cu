@@ -185,35 +185,58 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const ConvArgs a) {
   }
 }
 
-// ---------------------------------------------------------------- tcgen05 path (64 -> 64 layers)
-// The 64-channel convolutions run on the 5th-generation tensor cores.  One
-// thread is the producer and the MMA issuer: TMA (cp.async.bulk.tensor, 2-D
-// tensor map over the [K][64] BF16 activations) brings each tile's 142 input
-// rows (128 outputs + 14 halo rows, zero-filled beyond the sequence) into one
-// of three shared-memory stages, one group of 8 channels per box; a 1-D bulk
-// copy brings the packed weights once per CTA.  tcgen05.mma (M = 128 rows,
-// N = 64 channels, K = 16, BF16 in, FP32 accumulate in tensor memory) runs
-// 15 taps x 4 channel groups per tile from shared-memory descriptors in the
-// no-swizzle K-major layout: the box of a channel group is 142 rows of 16
-// bytes, so the operand for tap k is the same layout 16 k bytes further on
-// (no re-staging per tap).  Two TMEM accumulators let all four warps read
-// tile t back (tcgen05.ld, one row per thread) and apply bias + ReLU or the
-// ReLU mask of the layer below while tile t+1 computes and t+2 loads.
+// ---------------------------------------------------------------- tcgen05 path
+// All convolutions of the learned form on the 5th-generation tensor cores (BF16 in,
+// FP32 accumulate in tensor memory), one tile = 128 symbols (MMA M = 128 rows).
+//
+// 64 -> 64 layers (conv_tc_kernel): one persistent CTA per SM with all 15 weight
+// matrices (120 KB) in shared memory.  Warp 0 loads (TMA), warp 1 issues the MMAs,
+// warps 2-5 read the accumulators back and store; no CTA-wide barrier in the loop.
+// A tile's 142 input rows (128 + 14 halo, zero-filled beyond the sequence) arrive as one
+// box of 142 x 64 channels in the 128-byte-swizzled K-major layout, three stages deep;
+// the operand of tap k is the same box 128 k bytes further on.  The swizzle is what
+// makes that shift free: a row's 16-byte pieces sit in eight different bank groups
+// whatever row the operand starts at, while in the unswizzled layout (8 rows x 16 bytes
+// contiguous) a shift by k rows puts every core matrix across two 128-byte lines and
+// doubles the operand reads that bound an MMA of N = 64 (4 KB of A per 32 cycles of
+// math).  15 taps x 4 groups of 16 channels = 60 MMAs per tile into one of two
+// accumulators.  The output goes through swizzled shared memory to one TMA store per
+// warp (whole 128-byte rows, clipped at the sequence end).
+//
+// 4 -> 64 layers (edge_in_kernel: the first layer from the features, and dJ/dh of the
+// last one from dJ/dy): a feature row is 16 bytes of shared memory (4 values, 4 zeros), so
+// row n of tap k's operand is row n + k and the whole operand is again a shifted start;
+// the second half of K = 16 is a block of zeros that every operand shares through its
+// leading offset.  15 MMAs per tile, one per tap: the sums of the mma.sync form.
+// (Four taps per MMA on overlapping rows would take 4 MMAs, but rounds differently, and a
+// flipped BF16 rounding of one hidden value travels through every later layer.)
+//
+// 64 -> 4 layer (edge_out_kernel): the taps go to the N dimension instead,
+// P[m][4 t + c] = sum_ci h[m][ci] W[t][ci][c] (4 MMAs per tile, N = 64), and
+// out[n][c] = sum_t P[n + t - 7][4 t + c] is 15 float4 additions per symbol.  A tile of
+// 128 rows gives 114 symbols.  Both edge kernels are bound by the 128-byte rows they
+// write or read; several CTAs share an SM to overlap their phases.
 constexpr int TC_M = 128;                      // rows per tile (one MMA M)
 constexpr int TC_ROWS = TC_M + 2 * HALF;       // 142 rows per TMA box
-constexpr int TC_ROWS_P = 144;                 // group stride in rows (2304 B: 128-byte aligned)
-constexpr int TC_GROUPS = CH / 8;              // 8 groups of 8 channels (16 bytes)
 constexpr int TC_STAGES = 3;
-constexpr int TC_A_BYTES = TC_GROUPS * TC_ROWS_P * 16;   // 18432 per stage
-constexpr int TC_A_TX = TC_GROUPS * TC_ROWS * 16;        // 18176 bytes landed per stage
-constexpr int TC_W_BYTES = KS * TC_GROUPS * CH * 16;     // 122880: [tap][group][co][8]
-// + barriers, the TMEM address, and unused slack that keeps every operand read
-// inside the allocation even if a descriptor's two strides were read the other
-// way round (16 row groups x 2304 bytes past the last stage)
-constexpr int TC_SLACK = 38912;
-constexpr int TC_SMEM = TC_W_BYTES + TC_STAGES * TC_A_BYTES + 128 + TC_SLACK;
+constexpr int TC_A_BYTES = 18432;              // 144 rows x 128 B: stages stay 1024-byte aligned
+constexpr int TC_A_TX = TC_ROWS * 128;         // bytes landed per stage
+constexpr int TC_WCHUNKS = 3;                  // weights arrive in three pieces of 5 taps
+constexpr int TC_W_TAP = CH * CH * 2;          // 8192
+constexpr int TC_W_BYTES = KS * TC_W_TAP;      // 122880
+constexpr int TC_OUT_BYTES = TC_M * 128;       // 16384 per staging buffer
+constexpr int TC_OFF_A = TC_W_BYTES;
+constexpr int TC_OFF_OUT = TC_OFF_A + TC_STAGES * TC_A_BYTES;
+constexpr int TC_OFF_BIAS = TC_OFF_OUT + 2 * TC_OUT_BYTES;
+constexpr int TC_OFF_BAR = TC_OFF_BIAS + CH * 4;
+constexpr int TC_SMEM = TC_OFF_BAR + 256 + 1024;   // + slack to align the base to 1024 bytes
+constexpr int TC_THREADS = 192;
 constexpr unsigned TC_TMEM_COLS = 128;         // two accumulators of 64 FP32 columns
 constexpr long long kTcWaitNs = 2000000000ll;  // bounded waits
+
+constexpr int ED_W_BYTES = KS * CH * 16;       // weights of a 4 -> 64 layer: 16 bytes per tap and output
+constexpr int ED_TILE = TC_M - 2 * HALF;       // 114 symbols per tile of the 64 -> 4 layer
+constexpr unsigned ED_TMEM_COLS = 64;
 
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits
 // 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22,
@@ -221,12 +244,16 @@ constexpr long long kTcWaitNs = 2000000000ll;  // bounded waits
 constexpr unsigned TC_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(CH >> 3) << 17) |
                               ((unsigned)(TC_M >> 4) << 24);
 
-// Shared-memory matrix descriptor, no swizzle: start address, leading byte
-// offset (between core matrices adjacent in K) and stride byte offset (between
-// 8-row groups), all in 16-byte units; bits 46-47 = 1 (descriptor version).
+// Shared-memory matrix descriptor: start address, leading byte offset (no swizzle:
+// between core matrices adjacent in K) and stride byte offset (between 8-row groups), all
+// in 16-byte units; bits 46-47 = 1 (descriptor version); bits 61-63 the swizzle.
 __device__ __forceinline__ unsigned long long tc_desc(unsigned saddr, unsigned lbo, unsigned sbo) {
   return (unsigned long long)((saddr >> 4) & 0x3FFFu) | ((unsigned long long)((lbo >> 4) & 0x3FFFu) << 16) |
          ((unsigned long long)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+}
+// 128-byte swizzle, rows of 128 bytes, 8-row groups 1024 bytes apart
+__device__ __forceinline__ unsigned long long tc_desc_sw(unsigned saddr) {
+  return tc_desc(saddr, 16u, 1024u) | (2ull << 61);
 }
 
 __device__ __forceinline__ long long tc_now() {
@@ -235,7 +262,8 @@ __device__ __forceinline__ long long tc_now() {
   return t;
 }
 
-__device__ __forceinline__ bool tc_wait(unsigned mbar, unsigned parity, long long deadline) {
+// Bounded wait on an mbarrier phase; gives up past the deadline or once another role has.
+__device__ __forceinline__ bool tc_wait(unsigned mbar, unsigned parity, long long deadline, volatile int *fail) {
   for (;;) {
     unsigned done;
     asm volatile(
@@ -244,28 +272,72 @@ __device__ __forceinline__ bool tc_wait(unsigned mbar, unsigned parity, long lon
         : "r"(mbar), "r"(parity)
         : "memory");
     if (done) return true;
-    if (tc_now() > deadline) return false;
+    if (*fail) return false;
+    if (tc_now() > deadline) {
+      *fail = 1;
+      return false;
+    }
   }
 }
 
+// After a failure: a bounded wait (0.1 s) for a copy in flight.
+__device__ __forceinline__ void tc_drain(unsigned mbar, unsigned parity) {
+  int given_up = 0;
+  tc_wait(mbar, parity, tc_now() + 100000000ll, &given_up);
+}
+
+__device__ __forceinline__ void tc_bar_init(unsigned mbar, unsigned count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void tc_arrive(unsigned mbar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+}
 __device__ __forceinline__ void tc_expect(unsigned mbar, unsigned bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" :: "r"(mbar), "r"(bytes) : "memory");
 }
-
-// A tile: 8 boxes of (8 channels x 142 rows) at x = 8 g, y = n0 - 7 (negative or
-// past-the-end rows read as zero); x * 2 bytes is a multiple of 16.
-__device__ __forceinline__ void tc_load_tile(const CUtensorMap *tmap, unsigned stage_addr, int64_t n0, unsigned mbar) {
-  tc_expect(mbar, (unsigned)TC_A_TX);
-  const int y = (int)(n0 - HALF);
-#pragma unroll
-  for (int g = 0; g < TC_GROUPS; ++g) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
-        :: "r"(stage_addr + (unsigned)(g * TC_ROWS_P * 16)), "l"(reinterpret_cast<unsigned long long>(tmap)),
-           "r"(g * 8), "r"(y), "r"(mbar)
-        : "memory");
-  }
+__device__ __forceinline__ void tc_commit(unsigned mbar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar) : "memory");
 }
+__device__ __forceinline__ void tc_mma(unsigned d, unsigned long long a, unsigned long long b, bool acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+      :: "r"(d), "l"(a), "l"(b), "r"(TC_IDESC), "r"(acc ? 1u : 0u)
+      : "memory");
+}
+// 1-D bulk copy global -> shared (both 16-byte aligned)
+__device__ __forceinline__ void tc_bulk(unsigned dst, const void *src, unsigned bytes, unsigned mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+               :: "r"(dst), "l"(reinterpret_cast<unsigned long long>(src)), "r"(bytes), "r"(mbar)
+               : "memory");
+}
+// Box of 64 channels at row y (negative or past-the-end rows read as zero)
+__device__ __forceinline__ void tc_load_box(const CUtensorMap *tmap, unsigned dst, int64_t y, unsigned mbar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];\n"
+      :: "r"(dst), "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(0), "r"((int)y), "r"(mbar)
+      : "memory");
+}
+// Box of 32 rows x 64 channels to row y >= 0 (rows past the end are not written)
+__device__ __forceinline__ void tc_store_box(const CUtensorMap *tmap, unsigned src, int64_t y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];\n"
+               :: "l"(reinterpret_cast<unsigned long long>(tmap)), "r"(0), "r"((int)y), "r"(src)
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void tc_alloc(unsigned slot, unsigned cols) {
+  asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" :: "r"(slot), "r"(cols) : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+}
+__device__ __forceinline__ void tc_dealloc(unsigned tmem, unsigned cols) {
+  asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(cols) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
+// Results of earlier kernels of the stream are visible after this (a launch with the
+// programmatic attribute may start while the one before it drains).
+__device__ __forceinline__ void tc_grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void tc_grid_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 __device__ __forceinline__ void tc_ld32(unsigned taddr, float (&v)[32]) {
   unsigned r[32];
@@ -281,159 +353,409 @@ __device__ __forceinline__ void tc_ld32(unsigned taddr, float (&v)[32]) {
   for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// EPI_RELU: out = relu(acc + bias); EPI_MASK: out = acc * [mask > 0].
+// This warp's 32 accumulator rows (one per lane, 64 channels) -> bias + ReLU (EPI_RELU) or
+// the mask of the layer below (EPI_MASK) -> BF16 -> the warp's 4 KB of swizzled staging.
 template <int EPI>
-__global__ void __launch_bounds__(128, 1) conv_tc_kernel(const __grid_constant__ CUtensorMap tmap, const ConvArgs a,
-                                                         const void *__restrict__ wimg, int *__restrict__ err) {
-  extern __shared__ __align__(1024) unsigned char tc_smem[];
-  unsigned char *const Wb = tc_smem;
-  unsigned char *const Ab0 = tc_smem + TC_W_BYTES;
-  // barriers: [0] weights, [1..3] stage full, [4..5] accumulator ready
-  unsigned long long *bars = reinterpret_cast<unsigned long long *>(tc_smem + TC_W_BYTES + TC_STAGES * TC_A_BYTES);
-  unsigned *tmem_slot = reinterpret_cast<unsigned *>(bars + 8);
-  volatile int *fail_flag = reinterpret_cast<volatile int *>(bars + 9);   // CTA-uniform failure
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const unsigned bar_w = smem_u32(&bars[0]);
-  auto bar_full = [&](int s) { return smem_u32(&bars[1 + s]); };
-  auto bar_mma = [&](int s) { return smem_u32(&bars[4 + s]); };
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n"
-                 :: "r"(smem_u32(tmem_slot)), "r"(TC_TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-  }
-  if (tid == 0) {
-    for (int i = 0; i < 6; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" :: "r"(smem_u32(&bars[i])) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-    *fail_flag = 0;
-  }
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-  const unsigned tmem = *tmem_slot;
-  const unsigned wb_addr = smem_u32(Wb), ab_addr0 = smem_u32(Ab0);
-  const long long deadline = tc_now() + kTcWaitNs;
-  const int64_t n_tiles = (a.K + TC_M - 1) / TC_M;
-  const int64_t step = gridDim.x;
-  if (tid == 0) {
-    asm volatile("prefetch.tensormap [%0];\n" :: "l"(reinterpret_cast<unsigned long long>(&tmap)) : "memory");
-    tc_expect(bar_w, (unsigned)TC_W_BYTES);
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                 :: "r"(wb_addr), "l"(reinterpret_cast<unsigned long long>(wimg)), "r"((unsigned)TC_W_BYTES),
-                    "r"(bar_w)
-                 : "memory");
-    for (int s = 0; s < 2; ++s) {
-      const int64_t tile = blockIdx.x + s * step;
-      if (tile < n_tiles) tc_load_tile(&tmap, ab_addr0 + s * TC_A_BYTES, tile * TC_M, bar_full(s));
-    }
-  }
-  auto epilogue = [&](int64_t tile, int it) {
-    const int slot = it & 1;
-    if (!tc_wait(bar_mma(slot), (unsigned)((it >> 1) & 1), deadline)) {
-      *fail_flag = 1;
-      return;
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    float acc[64];
-    {
-      float v0[32], v1[32];
-      const unsigned taddr = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)(slot * 64);
-      tc_ld32(taddr, v0);
-      tc_ld32(taddr + 32, v1);
-      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+__device__ __forceinline__ void tc_store_rows(unsigned taddr, const float *bias, const uint4 (&mk)[8], unsigned char *stage,
+                                              int lane) {
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        acc[i] = v0[i];
-        acc[32 + i] = v1[i];
-      }
-    }
-    const int64_t n = tile * TC_M + warp * 32 + lane;
-    if (n >= a.K) return;
-    uint4 *dst = reinterpret_cast<uint4 *>(a.out + n * CH);
+  for (int hv = 0; hv < 2; ++hv) {
+    float v[32];
+    tc_ld32(taddr + 32 * hv, v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      float v[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e) v[e] = acc[q * 8 + e];
-      if constexpr (EPI == EPI_RELU) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = fmaxf(v[e] + a.bias[q * 8 + e], 0.f);
-      } else {
-        const uint4 mw = reinterpret_cast<const uint4 *>(a.mask + n * CH)[q];
-        const bf16 *mk = reinterpret_cast<const bf16 *>(&mw);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = __bfloat162float(mk[e]) > 0.f ? v[e] : 0.f;
-      }
+    for (int q = 0; q < 4; ++q) {
+      const int p = 4 * hv + q;
       __nv_bfloat162 o[4];
+      if constexpr (EPI == EPI_RELU) {
+        const float4 b0 = *reinterpret_cast<const float4 *>(bias + p * 8), b1 = *reinterpret_cast<const float4 *>(bias + p * 8 + 4);
+        o[0] = __floats2bfloat162_rn(fmaxf(v[8 * q] + b0.x, 0.f), fmaxf(v[8 * q + 1] + b0.y, 0.f));
+        o[1] = __floats2bfloat162_rn(fmaxf(v[8 * q + 2] + b0.z, 0.f), fmaxf(v[8 * q + 3] + b0.w, 0.f));
+        o[2] = __floats2bfloat162_rn(fmaxf(v[8 * q + 4] + b1.x, 0.f), fmaxf(v[8 * q + 5] + b1.y, 0.f));
+        o[3] = __floats2bfloat162_rn(fmaxf(v[8 * q + 6] + b1.z, 0.f), fmaxf(v[8 * q + 7] + b1.w, 0.f));
+      } else {
+        const bf16 *m = reinterpret_cast<const bf16 *>(&mk[p]);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) o[e] = __floats2bfloat162_rn(v[2 * e], v[2 * e + 1]);
-      dst[q] = *reinterpret_cast<uint4 *>(o);
-    }
-  };
-  int it = 0;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += step, ++it) {
-    // every read of the accumulator this tile overwrites (tile it - 2) is done
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    if (*fail_flag) break;                       // uniform: read after the barrier
-    if (tid == 0) {
-      const int s = it % TC_STAGES;
-      bool ok = true;
-      if (it == 0) ok = tc_wait(bar_w, 0u, deadline);
-      ok = ok && tc_wait(bar_full(s), (unsigned)((it / TC_STAGES) & 1), deadline);
-      if (ok) {
-        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-        const unsigned dcol = tmem + (unsigned)((it & 1) * 64);
-        const unsigned abase = ab_addr0 + s * TC_A_BYTES;
-        for (int k = 0; k < KS; ++k) {
-#pragma unroll
-          for (int kp = 0; kp < CH / 16; ++kp) {
-            const unsigned long long ad = tc_desc(abase + (2 * kp) * (TC_ROWS_P * 16) + k * 16, TC_ROWS_P * 16, 128);
-            const unsigned long long bd = tc_desc(wb_addr + ((k * TC_GROUPS + 2 * kp) * CH) * 16, CH * 16, 128);
-            const unsigned acc_in = (k | kp) ? 1u : 0u;
-            asm volatile(
-                "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-                :: "r"(dcol), "l"(ad), "l"(bd), "r"(TC_IDESC), "r"(acc_in)
-                : "memory");
-          }
-        }
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n"
-                     :: "r"(bar_mma(it & 1)) : "memory");
-        // the stage of tile it + 2 last held tile it - 1: free once its MMAs are done
-        const int64_t t2 = tile + 2 * step;
-        if (t2 < n_tiles) {
-          if (it >= 1) ok = tc_wait(bar_mma((it - 1) & 1), (unsigned)(((it - 1) >> 1) & 1), deadline);
-          if (ok) tc_load_tile(&tmap, ab_addr0 + ((it + 2) % TC_STAGES) * TC_A_BYTES, t2 * TC_M, bar_full((it + 2) % TC_STAGES));
-        }
+        for (int e = 0; e < 4; ++e)
+          o[e] = __floats2bfloat162_rn(__bfloat162float(m[2 * e]) > 0.f ? v[8 * q + 2 * e] : 0.f,
+                                       __bfloat162float(m[2 * e + 1]) > 0.f ? v[8 * q + 2 * e + 1] : 0.f);
       }
-      if (!ok) *fail_flag = 1;
+      *reinterpret_cast<uint4 *>(stage + lane * 128 + ((p ^ (lane & 7)) << 4)) = *reinterpret_cast<uint4 *>(o);
     }
-    __syncwarp();
-    if (it >= 1) epilogue(tile - step, it - 1);
-  }
-  __syncthreads();
-  if (!*fail_flag && it >= 1) epilogue(blockIdx.x + (int64_t)(it - 1) * step, it - 1);
-  __syncthreads();
-  if (*fail_flag && tid == 0) atomicExch(err, 1);
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-  __syncthreads();
-  if (warp == 0) {
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" :: "r"(tmem), "r"(TC_TMEM_COLS) : "memory");
   }
 }
 
-// Shared-memory image of one 64 -> 64 layer's weights for the tcgen05 path:
-// img[k][g][co][e] = Wsrc(k, ci = 8 g + e, co), with Wsrc the forward weights
-// W[k][ci][co] (rev = 0) or the input-gradient weights W[14 - k][co][ci] (rev = 1).
-__global__ void pack_tc_kernel(const float *__restrict__ W, bf16 *__restrict__ img, int rev) {
-  const int n = KS * CH * CH;
+// EPI_RELU: out = relu(acc + bias); EPI_MASK: out = acc * [mask > 0].
+template <int EPI>
+__global__ void __launch_bounds__(TC_THREADS, 1) conv_tc_kernel(const __grid_constant__ CUtensorMap tin,
+                                                                const __grid_constant__ CUtensorMap tout,
+                                                                const ConvArgs a, const void *__restrict__ wimg,
+                                                                int *__restrict__ err) {
+  extern __shared__ unsigned char tc_raw[];
+  unsigned char *const sm = tc_raw + ((1024u - (smem_u32(tc_raw) & 1023u)) & 1023u);
+  float *const bias = reinterpret_cast<float *>(sm + TC_OFF_BIAS);
+  unsigned long long *const bars = reinterpret_cast<unsigned long long *>(sm + TC_OFF_BAR);
+  unsigned *const tmem_slot = reinterpret_cast<unsigned *>(bars + 16);
+  volatile int *const fail = reinterpret_cast<volatile int *>(bars + 17);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto bar_w = [&](int i) { return smem_u32(&bars[i]); };
+  auto bar_full = [&](int s) { return smem_u32(&bars[3 + s]); };     // tile rows landed
+  auto bar_free = [&](int s) { return smem_u32(&bars[6 + s]); };     // their MMAs done
+  auto bar_acc = [&](int s) { return smem_u32(&bars[9 + s]); };      // accumulator complete
+  auto bar_read = [&](int s) { return smem_u32(&bars[11 + s]); };    // accumulator read back
+  if (warp == 1) tc_alloc(smem_u32(tmem_slot), TC_TMEM_COLS);
+  if (tid == 0) {
+    for (int i = 0; i < 11; ++i) tc_bar_init(smem_u32(&bars[i]), 1u);
+    for (int s = 0; s < 2; ++s) tc_bar_init(bar_read(s), 4u);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    *fail = 0;
+  }
+  if (EPI == EPI_RELU && tid < CH) bias[tid] = a.bias[tid];
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = *tmem_slot;
+  const unsigned w_addr = smem_u32(sm), a_addr = smem_u32(sm + TC_OFF_A);
+  const long long deadline = tc_now() + kTcWaitNs;
+  const int64_t n_tiles = (a.K + TC_M - 1) / TC_M;
+  const int64_t step = gridDim.x;
+  if (warp == 0) {
+    if (lane == 0) {
+      asm volatile("prefetch.tensormap [%0];\n" :: "l"(reinterpret_cast<unsigned long long>(&tin)) : "memory");
+      // the weights come from before the kernel in front of this one: no wait
+      for (int i = 0; i < TC_WCHUNKS; ++i) {
+        tc_expect(bar_w(i), (unsigned)(TC_W_BYTES / TC_WCHUNKS));
+        tc_bulk(w_addr + i * (TC_W_BYTES / TC_WCHUNKS),
+                static_cast<const unsigned char *>(wimg) + i * (TC_W_BYTES / TC_WCHUNKS),
+                (unsigned)(TC_W_BYTES / TC_WCHUNKS), bar_w(i));
+      }
+      tc_grid_wait();
+      // the next kernel may start its prologue on SMs that run out of tiles; everything
+      // before the kernel in front of this one is complete, so its weights are there
+      tc_grid_trigger();
+      int it = 0;
+      for (int64_t tile = blockIdx.x; tile < n_tiles; tile += step, ++it) {
+        const int s = it % TC_STAGES, round = it / TC_STAGES;
+        if (round > 0 && !tc_wait(bar_free(s), (unsigned)((round - 1) & 1), deadline, fail)) break;
+        tc_expect(bar_full(s), (unsigned)TC_A_TX);
+        tc_load_box(&tin, a_addr + s * TC_A_BYTES, tile * TC_M - HALF, bar_full(s));
+      }
+      if (*fail) {   // no copy left in flight
+        for (int i = 0; i < TC_WCHUNKS; ++i) tc_drain(bar_w(i), 0u);
+        for (int i = max(0, it - TC_STAGES); i < it; ++i) tc_drain(bar_full(i % TC_STAGES), (unsigned)((i / TC_STAGES) & 1));
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const unsigned long long a0 = tc_desc_sw(a_addr), w0 = tc_desc_sw(w_addr);
+      int it = 0;
+      bool ok = true;
+      for (int64_t tile = blockIdx.x; ok && tile < n_tiles; tile += step, ++it) {
+        const int s = it % TC_STAGES, acc = it & 1;
+        if (it >= 2) ok = tc_wait(bar_read(acc), (unsigned)(((it >> 1) - 1) & 1), deadline, fail);
+        ok = ok && tc_wait(bar_full(s), (unsigned)((it / TC_STAGES) & 1), deadline, fail);
+        if (!ok) break;
+        tc_fence_after();
+        const unsigned d = tmem + (unsigned)(acc * 64);
+        // every descriptor is a base plus a constant (the address field counts 16 bytes): with
+        // them built per MMA the one issuing thread is the bound (107 cycles per MMA
+        // whatever N; 48, the operand reads, as written)
+        const unsigned long long ad = a0 + (unsigned)(s * (TC_A_BYTES >> 4));
+#pragma unroll
+        for (int wc = 0; wc < TC_WCHUNKS; ++wc) {
+          if (it == 0 && ok) ok = tc_wait(bar_w(wc), 0u, deadline, fail);
+#pragma unroll
+          for (int i = 0; i < KS / TC_WCHUNKS * 4; ++i) {
+            const int k = wc * (KS / TC_WCHUNKS) + i / 4, kp = i % 4;
+            tc_mma(d, ad + (unsigned)(k * 8 + kp * 2), w0 + (unsigned)(k * (TC_W_TAP >> 4) + kp * 2), (k | kp) != 0);
+          }
+        }
+        tc_commit(bar_free(s));
+        tc_commit(bar_acc(acc));
+      }
+    }
+  } else {
+    const int quad = warp & 3;                  // the TMEM lanes this warp may read
+    tc_grid_wait();                             // the mask, and earlier readers of `out`
+    int it = 0;
+    for (int64_t tile = blockIdx.x; tile < n_tiles; tile += step, ++it) {
+      const int acc = it & 1;
+      const int64_t n0 = tile * TC_M + quad * 32;
+      uint4 mk[8];
+      if constexpr (EPI == EPI_MASK) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(a.mask + (n0 + lane) * CH);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) mk[q] = n0 + lane < a.K ? __ldg(&src[q]) : make_uint4(0u, 0u, 0u, 0u);
+      }
+      if (!tc_wait(bar_acc(acc), (unsigned)((it >> 1) & 1), deadline, fail)) break;
+      tc_fence_after();
+      unsigned char *stage = sm + TC_OFF_OUT + acc * TC_OUT_BYTES + quad * 4096;
+      // the store that last read this staging buffer (two tiles ago) is done with it
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+      __syncwarp();
+      tc_store_rows<EPI>(tmem + ((unsigned)(quad * 32) << 16) + (unsigned)(acc * 64), bias, mk, stage, lane);
+      tc_fence_before();
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      __syncwarp();
+      if (lane == 0) {
+        tc_arrive(bar_read(acc));
+        if (n0 < a.K) tc_store_box(&tout, smem_u32(stage), n0);
+        else asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+      }
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+    __syncwarp();
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && *fail) atomicExch(err, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tc_dealloc(tmem, TC_TMEM_COLS);
+  }
+}
+
+// 4 -> 64: SRC_Z from the received symbols (two pols, FP32), else from BF16 rows of FEATP.
+template <bool SRC_Z, int EPI>
+__global__ void __launch_bounds__(TC_M) edge_in_kernel(const __grid_constant__ CUtensorMap tout, const ConvArgs a,
+                                                       const void *__restrict__ wimg, int *__restrict__ err) {
+  __shared__ alignas(1024) unsigned char stage[TC_OUT_BYTES];
+  // feature rows, the weights [tap][out][8], and the zeros behind both
+  __shared__ struct alignas(128) { uint4 y[TC_ROWS + 2]; unsigned char w[ED_W_BYTES]; uint4 zero[TC_M]; } op;
+  __shared__ alignas(16) float bias[CH];
+  __shared__ unsigned long long bars[2];
+  __shared__ unsigned tmem_slot;
+  __shared__ volatile int fail_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const unsigned bar_w = smem_u32(&bars[0]), bar_acc = smem_u32(&bars[1]);
+  volatile int *const fail = &fail_s;
+  if (warp == 0) tc_alloc(smem_u32(&tmem_slot), ED_TMEM_COLS);
+  if (tid == 0) {
+    tc_bar_init(bar_w, 1u);
+    tc_bar_init(bar_acc, 1u);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    fail_s = 0;
+    tc_expect(bar_w, (unsigned)ED_W_BYTES);
+    tc_bulk(smem_u32(op.w), wimg, (unsigned)ED_W_BYTES, bar_w);
+  }
+  if (EPI == EPI_RELU && tid < CH) bias[tid] = a.bias[tid];
+  op.zero[tid] = make_uint4(0u, 0u, 0u, 0u);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = tmem_slot;
+  const long long deadline = tc_now() + kTcWaitNs;
+  const int64_t n_tiles = (a.K + TC_M - 1) / TC_M;
+  tc_grid_wait();
+  if (tid == 0) tc_grid_trigger();
+  const unsigned long long y0 = tc_desc(smem_u32(op.y), smem_u32(op.zero) - smem_u32(op.y), 128u);
+  const unsigned long long w0 = tc_desc(smem_u32(op.w), smem_u32(op.zero) - smem_u32(op.w), 128u);
+  // feature row of symbol n as four BF16 (zero outside the sequence)
+  auto feat = [&](int64_t n) -> uint2 {
+    if (n < 0 || n >= a.K) return make_uint2(0u, 0u);
+    if constexpr (SRC_Z) {
+      const float2 p0 = __ldg(&a.z[n]), p1 = __ldg(&a.z[a.z_stride + n]);
+      const __nv_bfloat162 v0 = __floats2bfloat162_rn(p0.x, p0.y), v1 = __floats2bfloat162_rn(p1.x, p1.y);
+      return make_uint2(*reinterpret_cast<const unsigned *>(&v0), *reinterpret_cast<const unsigned *>(&v1));
+    } else {
+      return __ldg(reinterpret_cast<const uint2 *>(a.in + n * FEATP));
+    }
+  };
+  int it = 0;
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+    const int64_t n0 = tile * TC_M;
+    for (int m = tid; m < TC_ROWS; m += TC_M) {
+      const uint2 v = feat(n0 - HALF + m);
+      op.y[m] = make_uint4(v.x, v.y, 0u, 0u);
+    }
+    uint4 mk[8];
+    const int64_t n = n0 + tid;
+    if constexpr (EPI == EPI_MASK) {
+      const uint4 *src = reinterpret_cast<const uint4 *>(a.mask + n * CH);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) mk[q] = n < a.K ? __ldg(&src[q]) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    tc_fence_before();
+    __syncthreads();   // rows written, the accumulator of the last tile read
+    tc_fence_after();
+    if (tid == 0 && (it > 0 || tc_wait(bar_w, 0u, deadline, fail))) {
+      // one row (or tap) on in the address is 16 bytes less to the zeros
+#pragma unroll
+      for (int k = 0; k < KS; ++k)
+        tc_mma(tmem, y0 + k - ((unsigned long long)k << 16), w0 + k * CH - ((unsigned long long)(k * CH) << 16), k != 0);
+      tc_commit(bar_acc);
+    }
+    const bool ok = tc_wait(bar_acc, (unsigned)(it & 1), deadline, fail);
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");
+    __syncwarp();
+    if (ok) {
+      tc_fence_after();
+      tc_store_rows<EPI>(tmem + ((unsigned)(warp * 32) << 16), bias, mk, stage + warp * 4096, lane);
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
+    __syncwarp();
+    if (ok && lane == 0 && n0 + warp * 32 < a.K) tc_store_box(&tout, smem_u32(stage + warp * 4096), n0 + warp * 32);
+    if (__syncthreads_or(!ok)) break;
+  }
+  if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+  if (tid == 0 && *fail) tc_drain(bar_w, 0u);
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && *fail) atomicExch(err, 1);
+  if (warp == 0) {
+    tc_fence_after();
+    tc_dealloc(tmem, ED_TMEM_COLS);
+  }
+}
+
+// 64 -> 4 with the residual output and, in training, dJ/dy and the loss (EPI_LAST).
+constexpr int ED_OUT_A = 0, ED_OUT_W = TC_OUT_BYTES, ED_OUT_P = ED_OUT_W + CH * CH * 2;
+constexpr int ED_OUT_SMEM = ED_OUT_P + KS * TC_M * 16 + 1024;   // + slack to align the base
+__global__ void __launch_bounds__(TC_M) edge_out_kernel(const __grid_constant__ CUtensorMap tin, const ConvArgs a,
+                                                        const void *__restrict__ wimg, int *__restrict__ err) {
+  extern __shared__ unsigned char tc_raw[];
+  unsigned char *const sm = tc_raw + ((1024u - (smem_u32(tc_raw) & 1023u)) & 1023u);
+  float4 *const P = reinterpret_cast<float4 *>(sm + ED_OUT_P);   // [tap][row]
+  __shared__ unsigned long long bars[3];
+  __shared__ unsigned tmem_slot;
+  __shared__ volatile int fail_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const unsigned bar_w = smem_u32(&bars[0]), bar_full = smem_u32(&bars[1]), bar_acc = smem_u32(&bars[2]);
+  const unsigned a_addr = smem_u32(sm + ED_OUT_A), w_addr = smem_u32(sm + ED_OUT_W);
+  volatile int *const fail = &fail_s;
+  if (warp == 0) tc_alloc(smem_u32(&tmem_slot), ED_TMEM_COLS);
+  const int64_t n_tiles = (a.K + ED_TILE - 1) / ED_TILE;
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i) tc_bar_init(smem_u32(&bars[i]), 1u);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    fail_s = 0;
+    tc_expect(bar_w, (unsigned)(CH * CH * 2));
+    tc_bulk(w_addr, wimg, (unsigned)(CH * CH * 2), bar_w);
+  }
+  float4 bias = make_float4(a.bias[0], a.bias[1], a.bias[2], a.bias[3]);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = tmem_slot;
+  const long long deadline = tc_now() + kTcWaitNs;
+  tc_grid_wait();
+  if (tid == 0) tc_grid_trigger();
+  if (tid == 0 && blockIdx.x < n_tiles) {
+    tc_expect(bar_full, (unsigned)TC_OUT_BYTES);
+    tc_load_box(&tin, a_addr, (int64_t)blockIdx.x * ED_TILE - HALF, bar_full);
+  }
+  double loss_part = 0.0;
+  int it = 0;
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, ++it) {
+    const int64_t n0 = tile * ED_TILE, n = n0 + tid;
+    const bool act = tid < ED_TILE && n < a.K;
+    float2 z0 = make_float2(0.f, 0.f), z1 = z0, t0 = z0, t1 = z0;
+    if (act) {
+      z0 = a.z[n];   // y may be z itself
+      z1 = a.z[a.z_stride + n];
+      if (a.t) {
+        t0 = __ldg(&a.t[n]);
+        t1 = __ldg(&a.t[a.t_stride + n]);
+      }
+    }
+    // the accumulator of the last tile is read (the barrier at the loop's end)
+    if (tid == 0 && (it > 0 || tc_wait(bar_w, 0u, deadline, fail)) &&
+        tc_wait(bar_full, (unsigned)(it & 1), deadline, fail)) {
+      tc_fence_after();
+#pragma unroll
+      for (int kp = 0; kp < 4; ++kp) tc_mma(tmem, tc_desc_sw(a_addr + kp * 32), tc_desc_sw(w_addr + kp * 32), kp != 0);
+      tc_commit(bar_acc);
+    }
+    const bool ok = tc_wait(bar_acc, (unsigned)(it & 1), deadline, fail);
+    if (ok) {
+      tc_fence_after();
+      if (tid == 0 && tile + gridDim.x < n_tiles) {      // the rows are consumed: the next tile's
+        tc_expect(bar_full, (unsigned)TC_OUT_BYTES);
+        tc_load_box(&tin, a_addr, (tile + gridDim.x) * ED_TILE - HALF, bar_full);
+      }
+      __syncwarp();
+#pragma unroll
+      for (int hv = 0; hv < 2; ++hv) {
+        float v[32];
+        tc_ld32(tmem + ((unsigned)(warp * 32) << 16) + 32 * hv, v);
+        asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+          if (8 * hv + t < KS) P[(8 * hv + t) * TC_M + tid] = make_float4(v[4 * t], v[4 * t + 1], v[4 * t + 2], v[4 * t + 3]);
+      }
+    }
+    tc_fence_before();
+    if (__syncthreads_or(!ok)) break;
+    tc_fence_after();
+    if (act) {
+      float4 s = P[tid];
+#pragma unroll
+      for (int t = 1; t < KS; ++t) {
+        const float4 v = P[t * TC_M + tid + t];
+        s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+      }
+      const float2 y0 = make_float2(z0.x + (s.x + bias.x), z0.y + (s.y + bias.y));
+      const float2 y1 = make_float2(z1.x + (s.z + bias.z), z1.y + (s.w + bias.w));
+      if (a.y) {
+        a.y[n] = y0;
+        a.y[a.y_stride + n] = y1;
+      }
+      if (a.t) {
+        const float d0 = y0.x - t0.x, d1 = y0.y - t0.y, d2 = y1.x - t1.x, d3 = y1.y - t1.y;
+        loss_part += ((double)d0 * d0 + (double)d1 * d1) + ((double)d2 * d2 + (double)d3 * d3);
+        const __nv_bfloat162 o0 = __floats2bfloat162_rn(2.f * d0 * a.inv4k, 2.f * d1 * a.inv4k);
+        const __nv_bfloat162 o1 = __floats2bfloat162_rn(2.f * d2 * a.inv4k, 2.f * d3 * a.inv4k);
+        *reinterpret_cast<uint2 *>(a.dout + n * FEATP) =
+            make_uint2(*reinterpret_cast<const unsigned *>(&o0), *reinterpret_cast<const unsigned *>(&o1));
+      }
+    }
+    __syncthreads();   // P is rewritten by the next tile
+  }
+  if (tid == 0 && *fail) {
+    tc_drain(bar_w, 0u);
+    tc_drain(bar_full, (unsigned)(it & 1));
+    tc_drain(bar_full, (unsigned)((it + 1) & 1));
+  }
+  if (a.t) {
+    for (int o = 16; o >= 1; o >>= 1) loss_part += __shfl_xor_sync(0xffffffffu, loss_part, o);
+    if (lane == 0 && loss_part != 0.0) atomicAdd(a.loss, loss_part * (double)a.inv4k);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && *fail) atomicExch(err, 1);
+  if (warp == 0) {
+    tc_fence_after();
+    tc_dealloc(tmem, ED_TMEM_COLS);
+  }
+}
+
+// Where weight W[k][ci][co] of a layer sits in its tcgen05 operand images.
+// 64 -> 64: [tap][co][ci] rows of 128 bytes, 16-byte pieces swizzled by row.
+__device__ __forceinline__ int img_sw(int row, int col) { return row * CH + (((col >> 3) ^ (row & 7)) << 3) + (col & 7); }
+__device__ __forceinline__ int img_tc_f(int k, int ci, int co) { return k * CH * CH + img_sw(co, ci); }
+__device__ __forceinline__ int img_tc_b(int k, int ci, int co) { return (KS - 1 - k) * CH * CH + img_sw(ci, co); }
+// 4 -> 64 (f: first layer, W[k][f][o]; b: reversed taps of the last layer, W[k][o][f]):
+// [tap][o][8], the upper four zero.
+__device__ __forceinline__ int img_in(int tap, int f, int o) { return (tap * CH + o) * 8 + f; }
+// 64 -> 4: rows 4 tap + c of 64 input channels, swizzled.
+__device__ __forceinline__ int img_out(int tap, int ci, int c) { return img_sw(4 * tap + c, ci); }
+
+// tcgen05 images of one layer from the master W[k][ci][co] (padding stays zero).
+__global__ void pack_tc_kernel(const float *__restrict__ W, int ci_true, int co_true, bf16 *__restrict__ f, bf16 *__restrict__ b) {
+  const int n = KS * ci_true * co_true;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const int k = i / (CH * CH), g = (i / (CH * 8)) % TC_GROUPS, co = (i / 8) % CH, e = i % 8;
-    const int ci = 8 * g + e;
-    const float v = rev ? W[((size_t)(KS - 1 - k) * CH + co) * CH + ci] : W[((size_t)k * CH + ci) * CH + co];
-    img[i] = __float2bfloat16_rn(v);
+    const int co = i % co_true, ci = (i / co_true) % ci_true, k = i / (co_true * ci_true);
+    const bf16 v = __float2bfloat16_rn(W[i]);
+    if (ci_true == FEAT) {
+      f[img_in(k, ci, co)] = v;
+    } else if (co_true == FEAT) {
+      f[img_out(k, ci, co)] = v;
+      b[img_in(KS - 1 - k, co, ci)] = v;
+    } else {
+      f[img_tc_f(k, ci, co)] = v;
+      b[img_tc_b(k, ci, co)] = v;
+    }
   }
 }
 
@@ -574,7 +896,7 @@ __global__ void features_kernel(const float2 *__restrict__ z, int64_t z_stride, 
 // written in the same pass (one launch per training step).
 struct PackLayer {
   long long off_w, off_b;
-  int ci, co, cinp, coutp, copb, tc;
+  int ci, co, cinp, coutp, copb;
   bf16 *wf, *wb, *wtc_f, *wtc_b;
 };
 struct PackTable {
@@ -602,9 +924,14 @@ __global__ void adam_pack_kernel(const PackTable tab, float *__restrict__ P, con
     const bf16 wv = __float2bfloat16_rn(w);
     y.wf[((size_t)k * y.coutp + co) * y.cinp + ci] = wv;
     if (y.wb) y.wb[((size_t)(KS - 1 - k) * y.ci + ci) * y.copb + co] = wv;
-    if (y.tc) {
-      y.wtc_f[(((size_t)k * TC_GROUPS + ci / 8) * CH + co) * 8 + ci % 8] = wv;
-      y.wtc_b[(((size_t)(KS - 1 - k) * TC_GROUPS + co / 8) * CH + ci) * 8 + co % 8] = wv;
+    if (y.ci == FEAT) {
+      y.wtc_f[img_in(k, ci, co)] = wv;
+    } else if (y.co == FEAT) {
+      y.wtc_f[img_out(k, ci, co)] = wv;
+      y.wtc_b[img_in(KS - 1 - k, co, ci)] = wv;
+    } else {
+      y.wtc_f[img_tc_f(k, ci, co)] = wv;
+      y.wtc_b[img_tc_b(k, ci, co)] = wv;
     }
   }
 }
@@ -653,7 +980,7 @@ struct rx_cnn {
   int sms = 0;
   float *P = nullptr, *G = nullptr, *M = nullptr, *V = nullptr;
   std::vector<bf16 *> wf, wb;
-  std::vector<bf16 *> wtc_f, wtc_b;    // tcgen05 shared-memory images of the 64 -> 64 layers
+  std::vector<bf16 *> wtc_f, wtc_b;    // tcgen05 operand images (wtc_b: none for the first layer)
   bool use_tc = true;
   int *err = nullptr;                  // sticky device error word (bounded waits)
   bf16 *x0 = nullptr, *dout = nullptr, *dza = nullptr, *dzb = nullptr;
@@ -757,24 +1084,69 @@ EncodeTiledFn encode_tiled() {
   return fn;
 }
 
-template <int EPI>
-cudaError_t launch_conv_tc(rx_cnn *c, const ConvArgs &a, const bf16 *img) {
-  KTimer tm(c, EPI == EPI_MASK ? RX_CNN_K_DX : RX_CNN_K_FWD_HIDDEN);
+// Tensor map of [K][64] BF16 rows in boxes of `rows` x 64 channels, 128-byte swizzle.
+cudaError_t row_map(CUtensorMap *m, const bf16 *p, int64_t K, unsigned rows) {
   EncodeTiledFn enc = encode_tiled();
   if (!enc) return cudaErrorNotSupported;
-  // [K][64] BF16 rows: dim 0 = channels (contiguous), dim 1 = symbols (128-byte stride)
-  CUtensorMap tmap;
-  const cuuint64_t dims[2] = {(cuuint64_t)CH, (cuuint64_t)a.K};
+  const cuuint64_t dims[2] = {(cuuint64_t)CH, (cuuint64_t)K};
   const cuuint64_t strides[1] = {(cuuint64_t)CH * sizeof(bf16)};
-  const cuuint32_t box[2] = {8u, (cuuint32_t)TC_ROWS};
+  const cuuint32_t box[2] = {(cuuint32_t)CH, rows};
   const cuuint32_t estr[2] = {1u, 1u};
-  if (enc(&tmap, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(a.in), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+  if (enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(p), dims, strides, box, estr,
+          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return cudaErrorInvalidValue;
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((a.K + TC_M - 1) / TC_M, c->sms));
-  conv_tc_kernel<EPI><<<grid, 128, TC_SMEM, c->stream>>>(tmap, a, img, c->err);
-  return cudaGetLastError();
+  return cudaSuccess;
+}
+
+// A launch that may start its prologue while the kernel in front of it drains (pdl).
+template <class... KArgs, class... Args>
+cudaError_t launch_tc(void (*fn)(KArgs...), int grid, int threads, int smem, cudaStream_t s, bool pdl, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
+int tc_grid(const rx_cnn *c, int64_t K, int tile, int per_sm) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((K + tile - 1) / tile, (int64_t)c->sms * per_sm));
+}
+
+template <int EPI>
+cudaError_t launch_conv_tc(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool pdl) {
+  KTimer tm(c, EPI == EPI_MASK ? RX_CNN_K_DX : RX_CNN_K_FWD_HIDDEN);
+  CUtensorMap tin, tout;
+  cudaError_t e = row_map(&tin, a.in, a.K, TC_ROWS);
+  if (e == cudaSuccess) e = row_map(&tout, a.out, a.K, 32);
+  if (e != cudaSuccess) return e;
+  return launch_tc(conv_tc_kernel<EPI>, tc_grid(c, a.K, TC_M, 1), TC_THREADS, TC_SMEM, c->stream, pdl, tin, tout, a,
+                   (const void *)img, c->err);
+}
+
+template <bool SRC_Z, int EPI>
+cudaError_t launch_edge_in(rx_cnn *c, const ConvArgs &a, const bf16 *img) {
+  KTimer tm(c, EPI == EPI_MASK ? RX_CNN_K_DX : RX_CNN_K_FWD_EDGE);
+  CUtensorMap tout;
+  const cudaError_t e = row_map(&tout, a.out, a.K, 32);
+  if (e != cudaSuccess) return e;
+  return launch_tc(edge_in_kernel<SRC_Z, EPI>, tc_grid(c, a.K, TC_M, 6), TC_M, 0, c->stream, false, tout, a,
+                   (const void *)img, c->err);
+}
+
+cudaError_t launch_edge_out(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool pdl) {
+  KTimer tm(c, RX_CNN_K_FWD_EDGE);
+  CUtensorMap tin;
+  const cudaError_t e = row_map(&tin, a.in, a.K, TC_M);
+  if (e != cudaSuccess) return e;
+  return launch_tc(edge_out_kernel, tc_grid(c, a.K, ED_TILE, 4), TC_M, ED_OUT_SMEM, c->stream, pdl, tin, a,
+                   (const void *)img, c->err);
 }
 
 template <int CIN, int COUT>
@@ -808,9 +1180,11 @@ rx_status check_sym(rx_cnn *c, const float *p, int64_t stride, int64_t K, const 
 
 // Forward pass; with t, also the loss and dJ/dy.  y may be NULL.
 rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, const float *t, int64_t ts, int64_t K) {
-  const int g = (int)std::min<int64_t>((K + 255) / 256, 4 * c->sms);
-  features_kernel<<<std::max(1, g), 256, 0, c->stream>>>(reinterpret_cast<const float2 *>(z), zs, K, c->x0);
-  CX_CUDA(cudaGetLastError(), "features");
+  if (t || !c->use_tc) {   // the feature rows: the weight gradient's input, and the mma.sync path's
+    const int g = (int)std::min<int64_t>((K + 255) / 256, 4 * c->sms);
+    features_kernel<<<std::max(1, g), 256, 0, c->stream>>>(reinterpret_cast<const float2 *>(z), zs, K, c->x0);
+    CX_CUDA(cudaGetLastError(), "features");
+  }
   const int L = c->L;
   for (int l = 0; l < L; ++l) {
     ConvArgs a;
@@ -819,20 +1193,22 @@ rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, c
     a.w = c->wf[l];
     a.bias = c->P + c->off_b[l];
     a.n_bias = c->co[l];
+    a.z = reinterpret_cast<const float2 *>(z);
+    a.z_stride = zs;
     if (l < L - 1) {
       a.in = l == 0 ? c->x0 : c->h[l - 1];
       a.out = c->h[l];
-      if (l == 0) {
+      if (l == 0 && c->use_tc) {
+        CX_CUDA((launch_edge_in<true, EPI_RELU>(c, a, c->wtc_f[l])), "conv (first)");
+      } else if (l == 0) {
         CX_CUDA((launch_conv<FEATP, CH, EPI_RELU>(c, a)), "conv");
       } else if (c->use_tc) {
-        CX_CUDA(launch_conv_tc<EPI_RELU>(c, a, c->wtc_f[l]), "conv (tensor memory)");
+        CX_CUDA(launch_conv_tc<EPI_RELU>(c, a, c->wtc_f[l], true), "conv (tensor memory)");
       } else {
         CX_CUDA((launch_conv<CH, CH, EPI_RELU>(c, a)), "conv");
       }
     } else {
       a.in = L == 1 ? c->x0 : c->h[L - 2];
-      a.z = reinterpret_cast<const float2 *>(z);
-      a.z_stride = zs;
       a.y = reinterpret_cast<float2 *>(y);
       a.y_stride = ys;
       a.t = reinterpret_cast<const float2 *>(t);
@@ -840,7 +1216,8 @@ rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, c
       a.dout = c->dout;
       a.loss = c->loss;
       a.inv4k = (float)(1.0 / (4.0 * (double)K));
-      CX_CUDA((launch_conv<CH, 8, EPI_LAST>(c, a)), "conv (last)");
+      if (c->use_tc) CX_CUDA(launch_edge_out(c, a, c->wtc_f[l], true), "conv (last)");
+      else CX_CUDA((launch_conv<CH, 8, EPI_LAST>(c, a)), "conv (last)");
     }
   }
   return RX_OK;
@@ -872,10 +1249,12 @@ rx_status backward(rx_cnn *c, int64_t K) {
     a.mask = c->h[l - 1];
     bf16 *out = bufs[l & 1];
     a.out = out;
-    if (last) {
+    if (last && c->use_tc) {
+      CX_CUDA((launch_edge_in<false, EPI_MASK>(c, a, c->wtc_b[l])), "input gradient");
+    } else if (last) {
       CX_CUDA((launch_conv<FEATP, CH, EPI_MASK>(c, a)), "input gradient");
     } else if (c->use_tc) {
-      CX_CUDA(launch_conv_tc<EPI_MASK>(c, a, c->wtc_b[l]), "input gradient (tensor memory)");
+      CX_CUDA(launch_conv_tc<EPI_MASK>(c, a, c->wtc_b[l], false), "input gradient (tensor memory)");
     } else {
       CX_CUDA((launch_conv<CH, CH, EPI_MASK>(c, a)), "input gradient");
     }
@@ -891,11 +1270,8 @@ rx_status pack(rx_cnn *c) {
     pack_kernel<<<64, 256, 0, c->stream>>>(c->P + c->off_w[l], c->ci[l], c->co[l], c->wf[l], cinp, coutp,
                                              l > 0 ? c->wb[l] : nullptr, copb);
     CX_CUDA(cudaGetLastError(), "pack");
-    if (l > 0 && l < c->L - 1) {
-      pack_tc_kernel<<<64, 256, 0, c->stream>>>(c->P + c->off_w[l], c->wtc_f[l], 0);
-      pack_tc_kernel<<<64, 256, 0, c->stream>>>(c->P + c->off_w[l], c->wtc_b[l], 1);
-      CX_CUDA(cudaGetLastError(), "pack (tensor memory)");
-    }
+    pack_tc_kernel<<<64, 256, 0, c->stream>>>(c->P + c->off_w[l], c->ci[l], c->co[l], c->wtc_f[l], c->wtc_b[l]);
+    CX_CUDA(cudaGetLastError(), "pack (tensor memory)");
   }
   return RX_OK;
 }
@@ -931,6 +1307,7 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   if (e == cudaSuccess) e = conv_prepare<CH, CH, EPI_MASK>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_kernel<EPI_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_kernel<EPI_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(edge_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ED_OUT_SMEM);
   if (e != cudaSuccess) {
     delete c;
     return RX_ECUDA;
@@ -950,9 +1327,10 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   c->wtc_f.assign(layers, nullptr);
   c->wtc_b.assign(layers, nullptr);
   CX_ALLOC(c->err, 1);
-  for (int l = 1; l < layers - 1; ++l) {
-    CX_ALLOC(c->wtc_f[l], (size_t)KS * CH * CH);
-    CX_ALLOC(c->wtc_b[l], (size_t)KS * CH * CH);
+  for (int l = 0; l < layers; ++l) {
+    const size_t n = l == 0 || l == layers - 1 ? (size_t)KS * CH * 8 : (size_t)KS * CH * CH;   // edges: at most
+    CX_ALLOC(c->wtc_f[l], n);
+    if (l > 0) CX_ALLOC(c->wtc_b[l], n);
   }
   for (int l = 0; l < layers; ++l) {
     const int cinp = l == 0 ? FEATP : CH, coutp = l == layers - 1 ? 8 : CH;
@@ -973,6 +1351,10 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   CX_CUDA(cudaMemset(c->V, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->dout, 0, K * FEATP * sizeof(bf16)), "init");   // channels 4..15 stay zero
   CX_CUDA(cudaMemset(c->err, 0, sizeof(int)), "init");
+  for (int l : {0, layers - 1}) {        // padding of the edge layers' images
+    CX_CUDA(cudaMemset(c->wtc_f[l], 0, (size_t)KS * CH * 8 * sizeof(bf16)), "init");
+    if (c->wtc_b[l]) CX_CUDA(cudaMemset(c->wtc_b[l], 0, (size_t)KS * CH * 8 * sizeof(bf16)), "init");
+  }
   rx_status s = pack(c);
   if (s != RX_OK) return s;
   CX_CUDA(cudaStreamSynchronize(c->stream), "create");
@@ -1082,7 +1464,6 @@ rx_status rx_cnn_train_step(rx_cnn *c, const float *z, int64_t zs, const float *
       y.copb = l == c->L - 1 ? FEATP : CH;
       y.wf = c->wf[l];
       y.wb = l > 0 ? c->wb[l] : nullptr;
-      y.tc = (l > 0 && l < c->L - 1) ? 1 : 0;
       y.wtc_f = c->wtc_f[l];
       y.wtc_b = c->wtc_b[l];
     }
