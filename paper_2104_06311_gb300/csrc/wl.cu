@@ -1,16 +1,17 @@
 // Four-tap widely-linear DD-LMS equaliser (declared in rx_wl.h).
 //
-// One thread runs one segment's symbols in order, everything in registers: the
-// taps as four real 2x2 matrices M_i = [[m00, m01], [m10, m11]] acting on
+// The taps are four real 2x2 matrices M_i = [[m00, m01], [m10, m11]] acting on
 // (Re u_i, Im u_i) -- the real form of h[i] u + g[i] conj(u), with
 // m00 = Re(h+g), m10 = Im(h+g), m11 = Re(h-g), m01 = -Im(h-g) -- so that the
 // output costs 16 FMAs and the LMS step M_i += 2 mu (Re e, Im e)^T (Re u, Im u)
-// another 16.  The strictly linear variant keeps h complex (g = 0).  Each warp
-// stages its 32 segments' inputs through shared memory in coalesced chunks,
-// one chunk ahead of the recursion.
-// Acquisition is the same code on one thread.  Decisions and the Gray bits
-// follow the dual-pol chain's rules; a thread's bits start on a word boundary
-// (segment starts are multiples of 16 symbols) and are written a word at a time.
+// another 16.  A segment's symbols run in order, everything in registers, on two
+// lanes (wl2_kernel: the two components of the output).  The strictly linear
+// variant keeps h complex (g = 0), which couples the components: one lane per segment
+// (wl_kernel).  Each warp stages its segments' inputs through shared memory in coalesced
+// chunks, one chunk ahead of the recursion.  Acquisition is the same code on one
+// segment.  Decisions and the Gray bits follow the dual-pol chain's rules; a segment's
+// bits start on a word boundary (segment starts are multiples of 16 symbols) and are
+// written a word at a time.
 #include <math.h>
 #include <string.h>
 
@@ -65,7 +66,7 @@ __device__ __forceinline__ float wl_decide(float v, unsigned &b) {
 // M(k-1) u(k) run beside the decision chain.  The strictly linear form keeps h
 // complex (m[i][0] = Re h, m[i][2] = Im h) with e' = mu e and the correction
 // e' sum conj(u_i(k-1)) u_i(k).
-template <int MB, bool LINEAR>
+template <int MB>
 struct WlRec {
   float m[WT][4];
   float u[WT][2];            // u_i = x[2k + c - i]: u0 = x[2k+1], u1 = x[2k], u2 = x[2k-1], u3 = x[2k-2]
@@ -78,69 +79,33 @@ struct WlRec {
     v[1][0] = p.x; v[1][1] = p.y;
     v[0][0] = p.z; v[0][1] = p.w;
     float r0 = 0.f, i0 = 0.f, r1 = 0.f, i1 = 0.f;
-    if (LINEAR) {
 #pragma unroll
-      for (int i = 0; i < WT; i += 2) {
-        r0 = fmaf(m[i][0], v[i][0], r0);
-        r0 = fmaf(-m[i][2], v[i][1], r0);
-        i0 = fmaf(m[i][0], v[i][1], i0);
-        i0 = fmaf(m[i][2], v[i][0], i0);
-        r1 = fmaf(m[i + 1][0], v[i + 1][0], r1);
-        r1 = fmaf(-m[i + 1][2], v[i + 1][1], r1);
-        i1 = fmaf(m[i + 1][0], v[i + 1][1], i1);
-        i1 = fmaf(m[i + 1][2], v[i + 1][0], i1);
-      }
-      // C = sum conj(u_i(k-1)) u_i(k)
-      float cr = 0.f, ci = 0.f;
+    for (int i = 0; i < WT; i += 2) {
+      r0 = fmaf(m[i][0], v[i][0], r0);
+      r0 = fmaf(-m[i][2], v[i][1], r0);
+      i0 = fmaf(m[i][0], v[i][1], i0);
+      i0 = fmaf(m[i][2], v[i][0], i0);
+      r1 = fmaf(m[i + 1][0], v[i + 1][0], r1);
+      r1 = fmaf(-m[i + 1][2], v[i + 1][1], r1);
+      i1 = fmaf(m[i + 1][0], v[i + 1][1], i1);
+      i1 = fmaf(m[i + 1][2], v[i + 1][0], i1);
+    }
+    // C = sum conj(u_i(k-1)) u_i(k)
+    float cr = 0.f, ci = 0.f;
 #pragma unroll
-      for (int i = 0; i < WT; ++i) {
-        cr = fmaf(u[i][0], v[i][0], cr);
-        cr = fmaf(u[i][1], v[i][1], cr);
-        ci = fmaf(u[i][0], v[i][1], ci);
-        ci = fmaf(-u[i][1], v[i][0], ci);
-      }
-      zr = fmaf(er, cr, fmaf(-ei, ci, r0 + r1));
-      zi = fmaf(er, ci, fmaf(ei, cr, i0 + i1));
-      // h_i += e' conj(u_i(k-1))
+    for (int i = 0; i < WT; ++i) {
+      cr = fmaf(u[i][0], v[i][0], cr);
+      cr = fmaf(u[i][1], v[i][1], cr);
+      ci = fmaf(u[i][0], v[i][1], ci);
+      ci = fmaf(-u[i][1], v[i][0], ci);
+    }
+    zr = fmaf(er, cr, fmaf(-ei, ci, r0 + r1));
+    zi = fmaf(er, ci, fmaf(ei, cr, i0 + i1));
+    // h_i += e' conj(u_i(k-1))
 #pragma unroll
-      for (int i = 0; i < WT; ++i) {
-        m[i][0] = fmaf(er, u[i][0], fmaf(ei, u[i][1], m[i][0]));
-        m[i][2] = fmaf(ei, u[i][0], fmaf(-er, u[i][1], m[i][2]));
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < WT; i += 2) {
-        r0 = fmaf(m[i][0], v[i][0], r0);
-        i0 = fmaf(m[i][2], v[i][0], i0);
-        r1 = fmaf(m[i + 1][0], v[i + 1][0], r1);
-        i1 = fmaf(m[i + 1][2], v[i + 1][0], i1);
-      }
-#pragma unroll
-      for (int i = 0; i < WT; i += 2) {
-        r0 = fmaf(m[i][1], v[i][1], r0);
-        i0 = fmaf(m[i][3], v[i][1], i0);
-        r1 = fmaf(m[i + 1][1], v[i + 1][1], r1);
-        i1 = fmaf(m[i + 1][3], v[i + 1][1], i1);
-      }
-      // c = u(k-1) . u(k), real
-      float c0 = 0.f, c1 = 0.f;
-#pragma unroll
-      for (int i = 0; i < WT; i += 2) {
-        c0 = fmaf(u[i][0], v[i][0], c0);
-        c0 = fmaf(u[i][1], v[i][1], c0);
-        c1 = fmaf(u[i + 1][0], v[i + 1][0], c1);
-        c1 = fmaf(u[i + 1][1], v[i + 1][1], c1);
-      }
-      const float c = c0 + c1;
-      zr = fmaf(er, c, r0 + r1);
-      zi = fmaf(ei, c, i0 + i1);
-#pragma unroll
-      for (int i = 0; i < WT; ++i) {
-        m[i][0] = fmaf(er, u[i][0], m[i][0]);
-        m[i][1] = fmaf(er, u[i][1], m[i][1]);
-        m[i][2] = fmaf(ei, u[i][0], m[i][2]);
-        m[i][3] = fmaf(ei, u[i][1], m[i][3]);
-      }
+    for (int i = 0; i < WT; ++i) {
+      m[i][0] = fmaf(er, u[i][0], fmaf(ei, u[i][1], m[i][0]));
+      m[i][2] = fmaf(ei, u[i][0], fmaf(-er, u[i][1], m[i][2]));
     }
 #pragma unroll
     for (int i = 0; i < WT; ++i) {
@@ -158,15 +123,8 @@ struct WlRec {
   __device__ __forceinline__ void flush() {
 #pragma unroll
     for (int i = 0; i < WT; ++i) {
-      if (LINEAR) {
-        m[i][0] = fmaf(er, u[i][0], fmaf(ei, u[i][1], m[i][0]));
-        m[i][2] = fmaf(ei, u[i][0], fmaf(-er, u[i][1], m[i][2]));
-      } else {
-        m[i][0] = fmaf(er, u[i][0], m[i][0]);
-        m[i][1] = fmaf(er, u[i][1], m[i][1]);
-        m[i][2] = fmaf(ei, u[i][0], m[i][2]);
-        m[i][3] = fmaf(ei, u[i][1], m[i][3]);
-      }
+      m[i][0] = fmaf(er, u[i][0], fmaf(ei, u[i][1], m[i][0]));
+      m[i][2] = fmaf(ei, u[i][0], fmaf(-er, u[i][1], m[i][2]));
     }
     er = ei = 0.f;
   }
@@ -184,7 +142,7 @@ constexpr int WSUB = 16;                 // symbols per sub-chunk: whole bit wor
 // ring, one chunk ahead of the recursion.  Chunks split into 16-symbol halves,
 // each entirely pretraining or entirely output (p0, s0 and S are multiples of
 // 16), so a full half runs unrolled with its bits gathered in registers.
-template <int MB, bool LINEAR, bool HAS_Z>
+template <int MB, bool HAS_Z>
 __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x4, int64_t K, int64_t s_begin,
                                                     int S, int nseg, int Wp, const WlTaps *__restrict__ taps_in,
                                                     WlTaps *__restrict__ taps_out, uint32_t *__restrict__ bits,
@@ -213,18 +171,16 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
     wl_cp_commit();
   };
   if (nch > 0) issue(0);
-  WlRec<MB, LINEAR> st;
+  WlRec<MB> st;
 #pragma unroll
   for (int i = 0; i < WT; ++i)
 #pragma unroll
     for (int q = 0; q < 4; ++q) st.m[i][q] = taps_in->m[i][q];
-  if (LINEAR) {
 #pragma unroll
-    for (int i = 0; i < WT; ++i) {   // keep h = (a + b)/2 as (m00, m10), drop g
-      const float hr = 0.5f * (st.m[i][0] + st.m[i][3]), hi = 0.5f * (st.m[i][2] - st.m[i][1]);
-      st.m[i][0] = hr;
-      st.m[i][2] = hi;
-    }
+  for (int i = 0; i < WT; ++i) {   // keep h = (a + b)/2 as (m00, m10), drop g
+    const float hr = 0.5f * (st.m[i][0] + st.m[i][3]), hi = 0.5f * (st.m[i][2] - st.m[i][1]);
+    st.m[i][0] = hr;
+    st.m[i][2] = hi;
   }
   // regressor history x[2 p0 - 1], x[2 p0 - 2]: before the buffer, the previous
   // buffer's last two samples; no pending update
@@ -236,7 +192,7 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
     st.u[0][0] = h.z; st.u[0][1] = h.w;   // x[2 p0 - 1]
   }
   st.er = st.ei = 0.f;
-  const float mu_s = LINEAR ? mu : 2.f * mu;
+  const float mu_s = mu;
   for (int c = 0; c < nch; ++c) {
     if (c + 1 < nch) {
       issue(c + 1);
@@ -292,12 +248,10 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
   }
   if (live && j == nseg - 1) {
     st.flush();
-    if (LINEAR) {
 #pragma unroll
-      for (int i = 0; i < WT; ++i) {
-        st.m[i][3] = st.m[i][0];
-        st.m[i][1] = -st.m[i][2];
-      }
+    for (int i = 0; i < WT; ++i) {
+      st.m[i][3] = st.m[i][0];
+      st.m[i][1] = -st.m[i][2];
     }
 #pragma unroll
     for (int i = 0; i < WT; ++i)
@@ -306,23 +260,244 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
   }
 }
 
-// one launch, modulation, form and the optional output as template arguments
-template <int MB, bool LINEAR>
-void launch_wl_mf(unsigned grid, cudaStream_t s, const float4 *x4, int64_t K, int64_t s_begin, int S, int nseg,
-                  int Wp, const WlTaps *tin, WlTaps *tout, uint32_t *bits, float2 *z, float mu, const float4 *tail) {
-  if (z)
-    wl_kernel<MB, LINEAR, true><<<grid, WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
-  else
-    wl_kernel<MB, LINEAR, false><<<grid, WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
+// Widely-linear form on two lanes per segment (16 segments per warp).  With M_i as above,
+// Re z and Im z are two recursions that share only their input: Re e updates the upper
+// rows (m00, m01) and Im e the lower ones, so lane `comp` of a pair runs component comp
+// with no exchange; every sum is formed in the order of a plain one-lane form.  A symbol is
+// one latency chain (correction, decision, error); the next symbol's dot product and the
+// tap update stand beside it, and a block's samples are read ahead.  One lane per segment
+// took 68 ns per symbol (561 us for the acquisition's 8192), four lanes with the taps
+// split as well 46 (their exchange waits on the chain), packed FP32 pairs 58, this form 41.
+// The segments of a warp run in lockstep over [s0 - W, s0 + S); where one starts later or
+// ends earlier its state holds.
+struct f2x { float x, y; };              // values of the taps i, i + 1
+__device__ __forceinline__ f2x f2_pack(float lo, float hi) { return f2x{lo, hi}; }
+__device__ __forceinline__ float f2_sum(f2x v) { return v.x + v.y; }
+__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) { return f2x{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) { return f2x{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
+
+// e' = mu_s (dec(z) - z) of one component and its Gray bits (wl_decide's).  Both levels'
+// errors are formed while |z| is compared: one select at the end of the chain.
+template <int MB>
+__device__ __forceinline__ float wl_error(float z, float mu_s, unsigned &b) {
+  const float mz = -mu_s * z;
+  if (MB == 2) {
+    const float d = wl_decide<2>(z, b);
+    return fmaf(mu_s, d, mz);
+  }
+  const bool outer = fabsf(z) > 0.63245553203367587f;      // |x sqrt 10| > 2
+  b = (z < 0.f ? 1u : 0u) | (outer ? 2u : 0u);
+  const bool pos = z >= 0.f;
+  const float e3 = fmaf(mu_s, pos ? 0.94868329805051381f : -0.94868329805051381f, mz);
+  const float e1 = fmaf(mu_s, pos ? 0.31622776601683793f : -0.31622776601683793f, mz);
+  return outer ? e3 : e1;
 }
 
-cudaError_t launch_wl(int mb, bool linear, unsigned grid, cudaStream_t s, const float4 *x4, int64_t K,
-                      int64_t s_begin, int S, int nseg, int Wp, const WlTaps *tin, WlTaps *tout, uint32_t *bits,
-                      float2 *z, float mu, const float4 *tail) {
-  if (mb == 2 && !linear) launch_wl_mf<2, false>(grid, s, x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
-  else if (mb == 2) launch_wl_mf<2, true>(grid, s, x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
-  else if (!linear) launch_wl_mf<4, false>(grid, s, x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
-  else launch_wl_mf<4, true>(grid, s, x4, K, s_begin, S, nseg, Wp, tin, tout, bits, z, mu, tail);
+template <int MB>
+struct WlRec2 {
+  f2x a01, a23, b01, b23;    // this component's row: factors of Re u (a) and Im u (b)
+  f2x r01, i01, r23, i23;    // Re, Im of the previous symbol's (u0, u1) and (u2, u3)
+  float e;                   // e' of the previous symbol (0 before the first)
+
+  // r = M(k-1) u(k) and c = u(k-1) . u(k); p = (x[2k], x[2k+1]) = (u1, u0)
+  __device__ __forceinline__ float dot(f2x vr, f2x vi) const {
+    f2x r = f2_mul(a01, vr);
+    r = f2_fma(a23, r01, r);
+    r = f2_fma(b01, vi, r);
+    r = f2_fma(b23, i01, r);
+    return f2_sum(r);
+  }
+  __device__ __forceinline__ float corr(f2x vr, f2x vi) const {
+    f2x c = f2_mul(r01, vr);
+    c = f2_fma(i01, vi, c);
+    c = f2_fma(r23, r01, c);
+    c = f2_fma(i23, i01, c);
+    return f2_sum(c);
+  }
+  __device__ __forceinline__ void shift(f2x vr, f2x vi) {
+    r23 = r01;
+    i23 = i01;
+    r01 = vr;
+    i01 = vi;
+  }
+
+  __device__ __forceinline__ float step(float4 p, float mu_s, unsigned &bit) {
+    const f2x vr = f2_pack(p.z, p.x), vi = f2_pack(p.w, p.y);
+    const float z = fmaf(e, corr(vr, vi), dot(vr, vi));
+    update();
+    shift(vr, vi);
+    e = wl_error<MB>(z, mu_s, bit);
+    return z;
+  }
+
+  // N symbols in order: the next symbol's sums in front of this one's decision.
+  template <int N, class F>
+  __device__ __forceinline__ void steps(const float4 *p, float mu_s, F emit) {
+    float4 x[N];
+#pragma unroll
+    for (int q = 0; q < N; ++q) x[q] = p[q];
+    f2x vr = f2_pack(x[0].z, x[0].x), vi = f2_pack(x[0].w, x[0].y);
+    float r = dot(vr, vi), c = corr(vr, vi);
+#pragma unroll
+    for (int q = 0; q < N; ++q) {
+      const float z = fmaf(e, c, r);
+      update();
+      shift(vr, vi);
+      if (q + 1 < N) {
+        vr = f2_pack(x[q + 1].z, x[q + 1].x);
+        vi = f2_pack(x[q + 1].w, x[q + 1].y);
+        r = dot(vr, vi);
+        c = corr(vr, vi);
+      }
+      unsigned b;
+      e = wl_error<MB>(z, mu_s, b);
+      emit(q, z, b);
+    }
+  }
+
+  __device__ __forceinline__ void update() {
+    const f2x ee = f2_pack(e, e);
+    a01 = f2_fma(ee, r01, a01);
+    a23 = f2_fma(ee, r23, a23);
+    b01 = f2_fma(ee, i01, b01);
+    b23 = f2_fma(ee, i23, b23);
+  }
+};
+
+constexpr int WSEG2 = WBLOCK / 2;        // segments per warp
+
+template <int MB, bool HAS_Z>
+__global__ void __launch_bounds__(WBLOCK) wl2_kernel(const float4 *__restrict__ x4, int64_t K, int64_t s_begin,
+                                                     int S, int nseg, int Wp, const WlTaps *__restrict__ taps_in,
+                                                     WlTaps *__restrict__ taps_out, uint32_t *__restrict__ bits,
+                                                     float2 *__restrict__ z, float mu, const float4 *__restrict__ tail) {
+  __shared__ __align__(16) float4 ring[2][WSEG2][WROW];
+  constexpr int WPS = WSUB * MB / 32;    // bit words per sub-chunk: 1 (QPSK) or 2 (16QAM)
+  const int lane = threadIdx.x;
+  const int seg = lane >> 1, comp = lane & 1;
+  const int j = blockIdx.x * WSEG2 + seg;
+  const bool live = j < nseg;
+  const int64_t s0 = s_begin + (int64_t)j * S;
+  const int64_t s1 = s0 + S < K ? s0 + S : K;
+  const int64_t base = s0 - Wp;          // symbol of the lockstep's first step
+  const int64_t p0 = base > 0 ? base : 0;
+  const int64_t b_first = s_begin + (int64_t)blockIdx.x * WSEG2 * S - Wp;   // base of the warp's segment 0
+  const int64_t span = (int64_t)Wp + S;
+  const int64_t nch = (span + WCH - 1) / WCH;
+  // chunk c of every segment: pairs base + c WCH + lane; zero outside the buffer or past the last segment
+  auto issue = [&](int64_t c) {
+#pragma unroll
+    for (int q = 0; q < WSEG2; ++q) {
+      const int64_t idx = b_first + (int64_t)q * S + c * WCH + lane;
+      const bool ok = blockIdx.x * WSEG2 + q < nseg && idx >= 0 && idx < K;
+      wl_cp16(&ring[c & 1][q][lane], ok ? (const void *)(x4 + idx) : (const void *)x4, ok ? 16 : 0);
+    }
+    wl_cp_commit();
+  };
+  issue(0);
+  WlRec2<MB> st;
+  st.a01 = f2_pack(taps_in->m[0][2 * comp], taps_in->m[1][2 * comp]);
+  st.a23 = f2_pack(taps_in->m[2][2 * comp], taps_in->m[3][2 * comp]);
+  st.b01 = f2_pack(taps_in->m[0][2 * comp + 1], taps_in->m[1][2 * comp + 1]);
+  st.b23 = f2_pack(taps_in->m[2][2 * comp + 1], taps_in->m[3][2 * comp + 1]);
+  st.r01 = st.i01 = st.r23 = st.i23 = f2_pack(0.f, 0.f);
+  st.e = 0.f;
+  if (live) {   // x[2 p0 - 1], x[2 p0 - 2]: before the buffer, the previous one's last two samples
+    const float4 h = p0 > 0 ? __ldg(&x4[p0 - 1]) : *tail;
+    st.r01 = f2_pack(h.z, h.x);
+    st.i01 = f2_pack(h.w, h.y);
+  }
+  const float mu_s = 2.f * mu;
+  for (int64_t c = 0; c < nch; ++c) {
+    if (c + 1 < nch) {
+      issue(c + 1);
+      wl_cp_wait<1>();
+    } else {
+      wl_cp_wait<0>();
+    }
+    __syncwarp();
+    const float4 *row = &ring[c & 1][seg][0];
+#pragma unroll 1
+    for (int h = 0; h < WCH / WSUB; ++h) {
+      const int64_t t0 = c * WCH + h * WSUB;               // the same for every segment
+      const int64_t start = base + t0;
+      const float4 *r = row + h * WSUB;
+      const bool out = t0 >= Wp;                           // Wp is a multiple of 16
+      const bool whole = !live || (start >= p0 && start + WSUB <= s1);
+      unsigned w[WPS];
+#pragma unroll
+      for (int t = 0; t < WPS; ++t) w[t] = 0u;
+      float *zo = HAS_Z ? reinterpret_cast<float *>(z + start) + comp : nullptr;
+      if (t0 >= span || !__any_sync(0xffffffffu, live && start < s1)) break;
+      if (__all_sync(0xffffffffu, whole)) {
+        st.template steps<WSUB>(r, mu_s, [&](int q, float zv, unsigned b) {
+          w[(q * MB) >> 5] |= b << ((q * MB) & 31);
+          if (HAS_Z && out && live) zo[2 * q] = zv;
+        });
+      } else {
+#pragma unroll 1
+        for (int q = 0; q < WSUB; ++q) {
+          unsigned b;
+          WlRec2<MB> nx = st;
+          const float zv = nx.step(r[q], mu_s, b);
+          if (live && start + q >= p0 && start + q < s1) {
+            st = nx;
+            if (MB == 2 || q < 8) w[0] |= b << ((q * MB) & 31);
+            else w[WPS - 1] |= b << ((q * MB) & 31);
+            if (HAS_Z && out) zo[2 * q] = zv;
+          }
+        }
+      }
+      if (out) {
+#pragma unroll
+        for (int t = 0; t < WPS; ++t) {
+          w[t] <<= comp * (MB / 2);
+          w[t] |= __shfl_xor_sync(0xffffffffu, w[t], 1);
+        }
+        const int64_t nv = s1 - start;
+        const int nw = (int)((min(nv, (int64_t)WSUB) * MB + 31) >> 5);
+        if (live && nv > 0 && comp < WPS && comp < nw) bits[((start * MB) >> 5) + comp] = comp == 0 ? w[0] : w[WPS - 1];
+      }
+    }
+    __syncwarp();   // the slot is refilled by the copy issued in the next iteration
+  }
+  wl_cp_wait<0>();
+  if (live && j == nseg - 1) {
+    st.update();    // the one still pending after the last symbol
+    const f2x row[4] = {st.a01, st.a23, st.b01, st.b23};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float lo = row[q].x, hi = row[q].y;
+      taps_out->m[2 * (q & 1)][2 * comp + (q >> 1)] = lo;
+      taps_out->m[2 * (q & 1) + 1][2 * comp + (q >> 1)] = hi;
+    }
+  }
+}
+
+// one launch, modulation, form and the optional output as template arguments
+template <int MB, bool LINEAR, bool HAS_Z>
+void launch_wl_k(cudaStream_t s, const float4 *x4, int64_t K, int64_t s_begin, int S, int nseg, int Wp, const WlTaps *tin,
+                 WlTaps *tout, uint32_t *bits, float2 *z, float mu, const float4 *tail) {
+  if constexpr (LINEAR)
+    wl_kernel<MB, HAS_Z><<<(unsigned)((nseg + WBLOCK - 1) / WBLOCK), WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout,
+                                                                                     bits, z, mu, tail);
+  else
+    wl2_kernel<MB, HAS_Z><<<(unsigned)((nseg + WSEG2 - 1) / WSEG2), WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout,
+                                                                                    bits, z, mu, tail);
+}
+
+template <int MB, bool LINEAR, class... Args>
+void launch_wl_z(bool has_z, Args... args) {
+  if (has_z) launch_wl_k<MB, LINEAR, true>(args...);
+  else launch_wl_k<MB, LINEAR, false>(args...);
+}
+
+template <class... Args>
+cudaError_t launch_wl(int mb, bool linear, bool has_z, Args... args) {
+  if (mb == 2 && !linear) launch_wl_z<2, false>(has_z, args...);
+  else if (mb == 2) launch_wl_z<2, true>(has_z, args...);
+  else if (!linear) launch_wl_z<4, false>(has_z, args...);
+  else launch_wl_z<4, true>(has_z, args...);
   return cudaGetLastError();
 }
 
@@ -521,8 +696,8 @@ rx_status rx_wl_process(rx_wl *w, const float *x, int64_t n, uint32_t *bits, flo
   if (!w->acquired) {
     a0 = std::min<int64_t>(w->A, K);
     if (a0 > 0) {
-      e = launch_wl(w->mb, w->linear, 1, w->stream, x4, K, 0, (int)a0, 1, 0, from, &w->dev[2], bits, z2,
-                    (float)w->mu, w->tail);
+      e = launch_wl(w->mb, w->linear, z2 != nullptr, w->stream, x4, K, (int64_t)0, (int)a0, 1, 0, from, &w->dev[2], bits, z2,
+                    (float)w->mu, (const float4 *)w->tail);
       from = &w->dev[2];
     }
     w->acquired = true;
@@ -532,9 +707,8 @@ rx_status rx_wl_process(rx_wl *w, const float *x, int64_t n, uint32_t *bits, flo
   const int nxt = 1 - w->cur;
   if (e == cudaSuccess && rest > 0) {
     const int64_t nseg = (rest + w->S - 1) / w->S;
-    const unsigned grid = (unsigned)((nseg + WBLOCK - 1) / WBLOCK);
-    e = launch_wl(w->mb, w->linear, grid, w->stream, x4, K, a0, w->S, (int)nseg, w->W, from, &w->dev[nxt], bits,
-                  z2, (float)w->mu, w->tail);
+    e = launch_wl(w->mb, w->linear, z2 != nullptr, w->stream, x4, K, a0, w->S, (int)nseg, w->W, from, &w->dev[nxt], bits,
+                  z2, (float)w->mu, (const float4 *)w->tail);
     w->cur = nxt;
   } else if (e == cudaSuccess && a0 > 0) {
     // the whole call was acquisition: its end taps start the next call
