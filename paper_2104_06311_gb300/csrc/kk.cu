@@ -2,16 +2,21 @@
 //
 // Stage 1 (kk_hilbert_kernel, one 64-thread CTA per two windows of 1024 samples,
 // hop 512, packed as real and imaginary parts of one transform): intensity I ->
-// a = sqrt(max(I, 1e-30)), ln a; radix-16 Stockham FFT
-// in shared memory; multiply by j sign(f) / N and conjugate; the same forward
-// FFT again gives the Hilbert image phi (inverse by conjugation); the kept
-// half of the window becomes E = a exp(j phi) exp(j 2 pi f_c n / fs), the
-// shift to DC taken from a 64-bit fixed-point phase accumulator.
-// Stage 2 (kk_filter_kernel, one 32-thread CTA per window): FFT 1024 of the
+// a = sqrt(max(I, 1e-30)), ln a (8-bit samples: a table of the 256 codes); FFT;
+// multiply by j sign(f) / N and conjugate; the same forward FFT again gives the
+// Hilbert image phi (inverse by conjugation); the kept half of the window becomes
+// E = a exp(j phi) exp(j 2 pi f_c n / fs), the shift to DC taken from a 64-bit
+// fixed-point phase accumulator.
+// Stage 2 (kk_filter_kernel, one 64-thread CTA per window): FFT 1024 of the
 // field, multiply by the static filter (dispersion inverse x RRC, with the 1/2
 // of the decimated DFT and 1/512 of the inverse folded in), keep the 512 bins
 // of |f| < fs/4, inverse 512-point FFT, keep the window's centre at 2 samples
 // per symbol.
+// Both stages hold a transform in the registers of 64 threads, element t + 64 i in
+// register i of thread t before and after every FFT: the last pass of the first
+// transform, the spectrum's multiplication and the first pass of the second work on the
+// same registers, the first and the last pass read and write global memory directly, and
+// the pair of FFTs crosses shared memory four times, one barrier each.
 #include <math.h>
 #include <string.h>
 
@@ -58,63 +63,148 @@ __device__ __forceinline__ float kk_intensity(const KkSrc &src, int64_t s) {
   return src.hist[s - (src.pos - KHIST)];
 }
 
+// ---- transforms of 64 threads: x[i] is element t + 64 i
+constexpr int KT = 64;
+constexpr int KBUF = KN + KN / 16;       // one float2 of padding per 16: unit- and 16-strided accesses conflict-free
+__device__ __forceinline__ int kpad(int i) { return i + (i >> 4); }
+
+// Stockham pass boundary: the R outputs of a pass of stride Ns (butterfly of inputs
+// t + 64 r) to buf; the next pass reads elements t + 64 i back.  With two buffers in turn a
+// thread is past the barrier of one exchange before any can write that buffer again; with
+// ONE buffer a barrier in front keeps the last exchange's reads ahead of the writes.
+template <int R, int Ns, int N, bool ONE = false>
+__device__ __forceinline__ void kk_exchange(float2 *buf, float2 (&x)[N / KT], int t) {
+  static_assert(R == N / KT, "one butterfly per thread");
+  const int d = (t / Ns) * Ns * R + (t & (Ns - 1));
+  if (ONE) __syncthreads();
+#pragma unroll
+  for (int r = 0; r < R; ++r) buf[kpad(d + r * Ns)] = x[r];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < R; ++i) x[i] = buf[kpad(t + KT * i)];
+}
+
+// x[r] *= W_{Ns R}^{r jm}
+template <int R, int Ns, int N>
+__device__ __forceinline__ void kk_twiddle(float2 (&x)[R], int jm, const float2 *__restrict__ tw) {
+  constexpr int TW = N / (Ns * R);
+#pragma unroll
+  for (int r = 1; r < R; ++r) x[r] = cmul(x[r], __ldg(&tw[r * jm * TW]));
+}
+
+// 1024-point forward FFT, radices 16, 16, 4 (the last as four butterflies j = t + 64 q of
+// elements j + 256 r, registers q + 4 r); natural order in and out.
+template <bool ONE>
+__device__ __forceinline__ void kk_fft1024(float2 (&x)[16], int t, float2 *b0, float2 *b1, const float2 *__restrict__ tw) {
+  dft<16>(x);
+  kk_exchange<16, 1, KN, ONE>(b0, x, t);
+  kk_twiddle<16, 16, KN>(x, t & 15, tw);
+  dft<16>(x);
+  kk_exchange<16, 16, KN, ONE>(b1, x, t);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    float2 v[4] = {x[q], x[q + 4], x[q + 8], x[q + 12]};
+    kk_twiddle<4, 256, KN>(v, t + KT * q, tw);
+    dft4(v[0], v[1], v[2], v[3]);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) x[q + 4 * r] = v[r];
+  }
+}
+
 // Windows 2b and 2b + 1 in one transform pair: window w gives the field of stream
 // samples [e0 + 512 w, e0 + 512 w + 512) from the input over [e0 + 512 w - 256,
 // e0 + 512 w + 768), written to E[s - e0].  The log-amplitudes of the two windows
 // are the real and imaginary parts of one complex sequence: the Hilbert response
 // j sign(f) maps real sequences to real ones, so the inverse transform returns the
 // first window's phase in its real part and the second's in its imaginary part --
-// two windows for the price of one FFT pair.
-__global__ void __launch_bounds__(KN / 16, 10) kk_hilbert_kernel(KkSrc src, int64_t e0, int nwin,
-                                                             const float2 *__restrict__ tw, unsigned long long inc_q,
-                                                             float2 *__restrict__ E) {
-  __shared__ float2 buf[KN + KN / 32];
+// two windows for the price of one FFT pair.  The second window is the first one 512
+// samples on, so a thread's samples t + 64 i (i < 24) serve both.
+// CTAs from n_pairs on copy the input history for the next buffer (hist_next): the
+// intensities of stream samples [pos + n - KHIST, pos + n).
+// Bound by instructions (two 1024-point FFTs, a sine and cosine per sample).
+template <bool I8>
+__global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e0, int nwin, int n_pairs,
+                                                            const float2 *__restrict__ tw, unsigned long long inc_q,
+                                                            float2 *__restrict__ E, float *__restrict__ hist_next) {
+  // one transform buffer: 12 CTAs per SM instead of 9
+  __shared__ float2 buf[KBUF];
+  __shared__ float2 lut[I8 ? 256 : 1];         // (ln a, a) of each code
+  __shared__ float amp[2 * KH];                // a of the kept samples, lo + 256 on
   const int t = threadIdx.x;
+  if ((int)blockIdx.x >= n_pairs) {
+    const int j = ((int)blockIdx.x - n_pairs) * KT + t;
+    if (j < KHIST) hist_next[j] = kk_intensity(src, src.pos + src.n - KHIST + j);   // before the stream start: never read
+    return;
+  }
+  if (I8) {
+    for (int c = t; c < 256; c += KT) {
+      const float p = fmaxf(((float)(c - 128) + src.offset) * src.scale, 1e-30f);
+      lut[c] = make_float2(0.5f * logf(p), sqrtf(p));
+    }
+    __syncthreads();
+  }
   const int w0 = 2 * blockIdx.x;
   const bool two = w0 + 1 < nwin;
-  const int64_t lo0 = e0 + (int64_t)w0 * KH - KH / 2, lo1 = lo0 + KH;
-  auto log_amp = [&](int64_t s) -> float {     // outside the stream: zero log-amplitude
-    return kk_inside(src, s) ? logf(sqrtf(fmaxf(kk_intensity(src, s), 1e-30f))) : 0.f;
+  const int64_t lo = e0 + (int64_t)w0 * KH - KH / 2;          // first sample of window w0
+  // every sample of both windows in the current buffer
+  const bool whole = two && lo >= src.pos && lo >= src.start && lo + KN + KH <= src.end;
+  const int8_t *in8 = reinterpret_cast<const int8_t *>(src.in) + (lo - src.pos);
+  const float *in32 = reinterpret_cast<const float *>(src.in) + (lo - src.pos);
+  auto sample = [&](int i) -> float2 {          // (ln a, a) of sample lo + i; (0, 0) outside the stream
+    const int64_t s = lo + i;
+    if (!whole && !kk_inside(src, s)) return make_float2(0.f, 0.f);
+    if (I8 && (whole || s >= src.pos)) return lut[(int)in8[i] + 128];
+    const float p = fmaxf(whole ? (in32[i] + src.offset) * src.scale : kk_intensity(src, s), 1e-30f);
+    return make_float2(0.5f * logf(p), sqrtf(p));
   };
-  for (int m = t; m < KN; m += blockDim.x)
-    buf[pad(m)] = make_float2(log_amp(lo0 + m), two ? log_amp(lo1 + m) : 0.f);
-  __syncthreads();
-  fft_forward<KN, 16>(buf, t, tw);
+  // a thread's samples through its own slots of the buffer: one copy of the sample code
+  float *const ln = reinterpret_cast<float *>(buf);
+#pragma unroll 4
+  for (int i = 0; i < 24; ++i) {
+    const int m = t + KT * i;
+    const float2 v = sample(m);
+    ln[m] = v.x;
+    if (i >= 4 && i < 20) amp[m - KH / 2] = v.y;
+  }
+  float2 x[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) x[i] = make_float2(ln[t + KT * i], two ? ln[t + KT * i + KH] : 0.f);
+  kk_fft1024<true>(x, t, buf, buf, tw);
   const float inv = 1.f / (float)KN;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const int k = t + q * (KN / 16);
-    const float2 v = buf[pad(k)];
-    float2 h;
-    if (k == 0 || k == KN / 2) h = make_float2(0.f, 0.f);
-    else if (k < KN / 2) h = make_float2(-v.y * inv, v.x * inv);     // x j
-    else h = make_float2(v.y * inv, -v.x * inv);                      // x (-j)
-    buf[pad(k)] = cconj(h);
+  for (int i = 0; i < 16; ++i) {                // conj(j sign(f) X / N): bins k = t + 64 i
+    const float2 v = x[i];
+    x[i] = i < 8 ? make_float2(-v.y * inv, -v.x * inv) : make_float2(v.y * inv, v.x * inv);
+    if (i % 8 == 0 && t == 0) x[i] = make_float2(0.f, 0.f);     // k = 0 and N / 2
   }
-  __syncthreads();
-  fft_forward<KN, 16>(buf, t, tw);
+  // the second transform forms its twiddles' addresses again: held from the first, they
+  // would spill
+  int t2 = t;
+  asm volatile("" : "+r"(t2));
+  kk_fft1024<true>(x, t2, buf, buf, tw);
   // inverse = conj of the forward transform of the conjugate: phase of window w0 in
   // the real part, of window w0 + 1 in the (negated) imaginary part
-  for (int i = t; i < 2 * KH; i += blockDim.x) {
-    const int w = i / KH, m = KH / 2 + (i % KH);
-    if (w == 1 && !two) break;
-    const int64_t s = e0 + (int64_t)(w0 + w) * KH + (m - KH / 2);
-    float2 e = make_float2(0.f, 0.f);            // outside the stream: zero field
-    if (kk_inside(src, s)) {
-      const float2 r = buf[pad(m)];
-      const float phi = w == 0 ? r.x : -r.y;
-      const float a = sqrtf(fmaxf(kk_intensity(src, s), 1e-30f));
-      float sp, cp;
-      sincosf(phi, &sp, &cp);
-      // exp(j 2 pi f_c s / fs) at stream sample s: the top 24 bits of the Q0.64 turn s inc_q
-      const unsigned long long ph = (unsigned long long)s * inc_q;
-      const float turns = (float)(ph >> 40) * 5.9604644775390625e-08f;   // 2^-24
-      float ss, cs;
-      sincospif(2.f * turns, &ss, &cs);
-      const float ex = a * cp, ey = a * sp;
-      e = make_float2(ex * cs - ey * ss, ex * ss + ey * cs);
-    }
-    E[s - e0] = e;
+  // (through the thread's own slots of the buffer)
+  float *const ph = ln;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    ph[t + KT * i] = x[i + 4].x;
+    ph[t + KT * i + KH] = -x[i + 4].y;
+  }
+  const int n_out = two ? 16 : 8;
+#pragma unroll 4
+  for (int i = 0; i < n_out; ++i) {
+    const int m = t + KT * i;                    // field sample of the pair
+    const int64_t s = lo + KH / 2 + m;
+    const float a = amp[m];                      // outside the stream: zero field
+    // exp(j (phi + 2 pi f_c s / fs)): the turn s inc_q (signed Q0.64) in half turns to 32
+    // bits, phi / pi in two terms, one sine and cosine
+    const float turn = (float)(int)(((unsigned long long)s * inc_q) >> 32) * 4.65661287307739258e-10f;   // 2^-31
+    const float phi = ph[m];
+    float sp, cp;
+    sincospif(fmaf(phi, 0.31830987334251404f, fmaf(phi, 1.2841276632e-08f, turn)), &sp, &cp);
+    E[s - e0] = make_float2(a * cp, a * sp);
   }
 }
 
@@ -122,47 +212,51 @@ __global__ void __launch_bounds__(KN / 16, 10) kk_hilbert_kernel(KkSrc src, int6
 // output samples t in [i S, i S + S) inside [o0, o0 + no) at 2 samples/symbol to
 // y[(t - o0)/2] (zero before the stream start); optionally the field itself to
 // field[t - o0] for every t of the range.
-__global__ void __launch_bounds__(32, 20) kk_filter_kernel(const float2 *__restrict__ E, int64_t e0, int64_t i0, int64_t o0,
+__global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *__restrict__ E, int64_t e0, int64_t i0, int64_t o0,
                                                        int64_t no, int64_t start, int V,
                                                        const float2 *__restrict__ H, const float2 *__restrict__ tw,
                                                        const float2 *__restrict__ tw2, float2 *__restrict__ y,
                                                        float2 *__restrict__ field) {
-  __shared__ float2 buf[KN + KN / 32];
-  __shared__ float2 buf2[KN2 + KN2 / 32];
+  __shared__ float2 b0[KBUF], b1[KBUF];
   const int t = threadIdx.x;
   const int S = KN - V;
   const int64_t i = i0 + blockIdx.x;
   const int64_t lo = i * S - V / 2;
-  for (int m = t; m < KN; m += 32) buf[pad(m)] = E[lo + m - e0];
-  __syncthreads();
+  float2 x[16];
+  const float2 *src = E + (lo - e0) + t;
+#pragma unroll
+  for (int q = 0; q < 16; ++q) x[q] = src[KT * q];
   if (field) {
-    for (int m = V / 2 + t; m < V / 2 + S; m += 32) {
+#pragma unroll
+    for (int q = 0; q < 16; ++q) {
+      const int m = t + KT * q;
       const int64_t tt = lo + m;
-      if (tt >= o0 && tt < o0 + no) field[tt - o0] = buf[pad(m)];
+      if (m >= V / 2 && m < V / 2 + S && tt >= o0 && tt < o0 + no) field[tt - o0] = x[q];
     }
   }
-  fft_forward<KN, 32>(buf, t, tw);
+  kk_fft1024<false>(x, t, b0, b1, tw);
   // keep |f| < fs/4: bins k < 256 -> k, k >= 768 -> k - 512; conjugate for the inverse
-  for (int k = t; k < KN; k += 32) {
-    if (k >= KN / 4 && k < KN - KN / 4) continue;
-    const int d = k < KN / 4 ? k : k - KN2;
-    buf2[pad(d)] = cconj(cmul(buf[pad(k)], __ldg(&H[k])));
+  float2 z[8];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int r = q < 4 ? q : q + 8;
+    z[q] = cconj(cmul(x[r], __ldg(&H[t + KT * r])));
   }
-  __syncthreads();
-  fft_forward<KN2, 16>(buf2, t, tw2);
-  for (int m = V / 4 + t; m < V / 4 + S / 2; m += 32) {
+  // 512-point forward FFT, radices 8, 8, 8
+  dft<8>(z);
+  kk_exchange<8, 1, KN2>(b0, z, t);
+  kk_twiddle<8, 8, KN2>(z, t & 7, tw2);
+  dft<8>(z);
+  kk_exchange<8, 8, KN2>(b1, z, t);
+  kk_twiddle<8, 64, KN2>(z, t, tw2);
+  dft<8>(z);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int m = t + KT * q;
     const int64_t tt = i * S + 2 * (m - V / 4);      // input-rate sample of this output
-    if (tt < o0 || tt >= o0 + no) continue;
-    y[(tt - o0) / 2] = tt >= start ? cconj(buf2[pad(m)]) : make_float2(0.f, 0.f);
+    if (m < V / 4 || m >= V / 4 + S / 2 || tt < o0 || tt >= o0 + no) continue;
+    y[(tt - o0) / 2] = tt >= start ? cconj(z[q]) : make_float2(0.f, 0.f);
   }
-}
-
-// History for the next buffer: intensities of stream samples [pos + n - KHIST, pos + n).
-__global__ void kk_hist_kernel(KkSrc src, float *__restrict__ next) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= KHIST) return;
-  const int64_t s = src.pos + src.n - KHIST + j;
-  next[j] = kk_intensity(src, s);   // entries before the stream start are never read
 }
 
 }  // namespace
@@ -314,19 +408,20 @@ rx_status kk_run(rx_kk *k, const KkSrc &src, int64_t no, float *y, float *field)
   const int64_t o0 = k->pos - KDELAY, e0 = o0 - KEDGE;
   if (ev[0]) cudaEventRecord(ev[0], k->stream);
   const int nwin = (int)((no + 2 * KEDGE) / KH);
-  kk_hilbert_kernel<<<(unsigned)((nwin + 1) / 2), KN / 16, 0, k->stream>>>(src, e0, nwin, k->tw, k->inc_q, k->E);
+  const int n_pairs = (nwin + 1) / 2;
+  const unsigned grid = (unsigned)(n_pairs + (src.n > 0 ? KHIST / KT : 0));   // + the history's copy
+  if (src.dtype == RX_KK_I8)
+    kk_hilbert_kernel<true><<<grid, KT, 0, k->stream>>>(src, e0, nwin, n_pairs, k->tw, k->inc_q, k->E, k->hist[1 - k->cur]);
+  else
+    kk_hilbert_kernel<false><<<grid, KT, 0, k->stream>>>(src, e0, nwin, n_pairs, k->tw, k->inc_q, k->E, k->hist[1 - k->cur]);
   cudaError_t e = cudaGetLastError();
   if (ev[1]) cudaEventRecord(ev[1], k->stream);
   const int S = KN - k->V;
   const int64_t i0 = floor_div(o0, S), i1 = floor_div(o0 + no - 1, S);
   if (e == cudaSuccess) {
-    kk_filter_kernel<<<(unsigned)(i1 - i0 + 1), 32, 0, k->stream>>>(
+    kk_filter_kernel<<<(unsigned)(i1 - i0 + 1), KT, 0, k->stream>>>(
         k->E, e0, i0, o0, no, k->start, k->V, k->H, k->tw, k->tw2, reinterpret_cast<float2 *>(y),
         reinterpret_cast<float2 *>(field));
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess && src.n > 0) {
-    kk_hist_kernel<<<(KHIST + 255) / 256, 256, 0, k->stream>>>(src, k->hist[1 - k->cur]);
     e = cudaGetLastError();
   }
   if (ev[2]) {

@@ -1,0 +1,27 @@
+"""Kramers-Kronig front end with the shortest buffers (odd and even window counts, buffers
+inside the look-ahead and the history) against the FP64 reference (oracle/kk.py), for the
+table-driven 8-bit form and the float one."""
+import pytest
+
+import linksim.kk as LK
+from oracle import kk as K
+from chain_helpers import rel_rms
+from test_gpu_kk import TOL, _built, _stream  # noqa: F401  (_built: module fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("adc", ["int8", "f32"])
+@pytest.mark.parametrize("bufs", [[1], [2], [1, 1, 1, 2, 3, 5], [7, 1, 2], [6, 4, 11]])
+def test_short_buffers(adc, bufs):
+    from paper_2104_06311_gb300 import KKFrontEnd
+    n = 512 * sum(bufs)
+    lk = LK.KKLink(n_sym=n // 4, adc=adc, L_km=1500.0, cspr_db=12.0, snr_db=24.0, seed=2104063151 + n)
+    g = LK.generate(lk)
+    cuts = [0]
+    for b in bufs:
+        cuts.append(cuts[-1] + 512 * b)
+    fe = KKFrontEnd(lk.baud, lk.carrier_hz, lk.L_km, 512 * max(bufs))
+    yg, fg = _stream(fe, g.samples, cuts, g)
+    yo, Eo, _ = K.kk_frontend(g.samples, g.in_scale, g.in_offset, lk.baud, lk.sps, lk.carrier_hz, lk.L_km)
+    assert rel_rms(fg, Eo) < TOL and rel_rms(yg, yo) < TOL
