@@ -298,9 +298,14 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_blk(BpsLaunch L) {
   }
 }
 
+// One CTA per pol.  A thread owns a run of chunks; the prefix over the 1024 threads goes
+// by warp shuffles and one pass over the 32 warp totals.  A region's noise variance is a
+// warp's sum over its chunks (lane-strided in double, then a butterfly).  Bound by the
+// latency of its loads; region sums by one thread each took 17.5 us of a call's tail at 128
+// chunks per region, the warps take 4.5.
 __global__ void __launch_bounds__(1024) bps_scan(BpsLaunch L) {
-  __shared__ int64_t part[1024];
-  const int p = blockIdx.x, t = threadIdx.x;
+  __shared__ int64_t part[32];
+  const int p = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int64_t n = L.n_chunks;
   const int64_t per = (n + 1023) / 1024;
   const int64_t c0 = min((int64_t)t * per, n), c1 = min(c0 + per, n);
@@ -314,36 +319,43 @@ __global__ void __launch_bounds__(1024) bps_scan(BpsLaunch L) {
     L.chunk_r[(int64_t)p * n + c] = r;
     s += r;
   }
-  part[t] = s;
-  __syncthreads();
-  // Hillis-Steele inclusive scan over 1024 partials
-  for (int o = 1; o < 1024; o <<= 1) {
-    int64_t v = t >= o ? part[t - o] : 0;
-    __syncthreads();
-    part[t] += v;
-    __syncthreads();
+  int64_t inc = s;                               // inclusive over the warp
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
   }
-  int64_t run = L.m_carry[p] + (t > 0 ? part[t - 1] : 0);
+  if (lane == 31) part[warp] = inc;
+  const int64_t carry = L.m_carry[p];
+  __syncthreads();
+  int64_t before = 0, total = 0;                 // chunks of earlier warps, of all
+#pragma unroll
+  for (int w = 0; w < 32; ++w) {
+    before += w < warp ? part[w] : 0;
+    total += part[w];
+  }
+  int64_t run = carry + before + (inc - s);
   for (int64_t c = c0; c < c1; ++c) {
     L.chunk_m[(int64_t)p * n + c] = run;
     run += L.chunk_r[(int64_t)p * n + c];
   }
-  __syncthreads();
-  if (t == 1023) L.m_carry[p] += part[1023];
+  if (t == 0) L.m_carry[p] = carry + total;      // every thread read it before the barrier
   if (!L.need_s2) return;   // sigma^2 feeds the LLRs only
   // regions: [0, A), then [A + r span, ...), clipped to [k_lo, k_hi) (calls emit whole
   // regions, so a region's chunks start at its first symbol)
   const int64_t r_lo = L.k_lo < L.A ? 0 : 1 + (L.k_lo - L.A) / L.span;
   const int64_t r_hi = L.k_hi <= L.A ? 1 : 1 + (L.k_hi - 1 - L.A) / L.span + 1;
-  for (int64_t r = r_lo + t; r < r_hi; r += 1024) {
+  for (int64_t r = r_lo + warp; r < r_hi; r += 32) {
     const int64_t s_r = r == 0 ? 0 : L.A + (r - 1) * L.span;
     const int64_t e_r = min(r == 0 ? L.A : s_r + L.span, L.k_hi);
-    const int64_t c0 = (s_r - L.k_lo) / L.chunk;
-    const int64_t c1 = min(n, (e_r - L.k_lo + L.chunk - 1) / L.chunk);   // chunks starting before e_r
+    const int64_t q0 = (s_r - L.k_lo) / L.chunk;
+    const int64_t q1 = min(n, (e_r - L.k_lo + L.chunk - 1) / L.chunk);   // chunks starting before e_r
     double acc = 0.0;
-#pragma unroll 8
-    for (int64_t c = c0; c < c1; ++c) acc += (double)L.chunk_s2[(int64_t)p * n + c];
-    L.region_s2[(int64_t)p * (r_hi - r_lo) + (r - r_lo)] = acc / (double)(e_r - s_r);
+#pragma unroll 4
+    for (int64_t c = q0 + lane; c < q1; c += 32) acc += (double)L.chunk_s2[(int64_t)p * n + c];
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) L.region_s2[(int64_t)p * (r_hi - r_lo) + (r - r_lo)] = acc / (double)(e_r - s_r);
   }
 }
 

@@ -30,6 +30,7 @@ using namespace rx;
 
 namespace {
 constexpr int kMaxPieces = 64;
+constexpr int kFineChunks = 2048;   // BPS chunks per pol below which a launch takes finer ones
 constexpr uint32_t kStateMagic = 0x52584231u;  // "RXB1"
 }  // namespace
 
@@ -316,6 +317,17 @@ unsigned char *u_at(rx_stream *rx, int b, int p, int64_t n) {
 }
 
 // Region layout: region 0 = [0, A), region r >= 1 = [A + (r-1) span, A + r span).
+// Symbols per BPS chunk (one warp each).  A chunk's pass is one chain of 32-symbol blocks
+// after a first block that fills its window, so with few chunks the launch lasts as long
+// as one of them: the chunk shrinks (by whole powers of two of C, so that regions still
+// start on one) while the launch stays below kFineChunks chunks per pol, about seven
+// warps per scheduler of both pols.
+int bps_chunk(const rx_stream *rx, int64_t n) {
+  int c = rx->C;
+  while (c > 64 && c % 64 == 0 && (n + c / 2 - 1) / (c / 2) <= kFineChunks) c /= 2;
+  return c;
+}
+
 int64_t region_end_after(const rx_stream *rx, int64_t k) {
   // end of the region that starts at or contains symbol k
   if (k < rx->A) return rx->A;
@@ -499,7 +511,7 @@ rx_status rx_reserve(rx_stream *rx, int64_t max_call) {
   // equaliser's bulk-copied window rows land 8 bytes apart in the shared-memory banks
   rx->u_cap |= 1;
   rx->y_cap = max_call / 2 + 4 * region + 4 * rx->Nb + 4096;
-  rx->chunk_cap = rx->y_cap / rx->C + 16;
+  rx->chunk_cap = rx->y_cap / rx->C + 16 + kFineChunks;
   rx->region_cap = rx->y_cap / std::min(rx->A_full > 0 ? rx->A_full : rx->span, rx->span) + 16;
 #define RX_ALLOC(ptr, count)              \
   do {                                    \
@@ -808,8 +820,8 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       B.bhat = rx->bh[rx->cur_y];
       B.bh_base = rx->y_base;
       B.bh_stride = rx->y_cap;
-      B.chunk = rx->C;
-      B.n_chunks = (kj - kdone + rx->C - 1) / rx->C;
+      B.chunk = bps_chunk(rx, kj - kdone);
+      B.n_chunks = (kj - kdone + B.chunk - 1) / B.chunk;
       if (B.n_chunks > rx->chunk_cap) return fail(rx, RX_EINVAL, "chunk table overflow");
       B.chunk_r = rx->chunk_r;
       B.chunk_s2 = rx->chunk_s2;
