@@ -96,6 +96,7 @@ struct rx_stream {
   int eq_alt_ok = 0;                // 4 P CTAs fit co-resident
   int sms = 0;                      // multiprocessors of the device
   int pieces = 12;                  // pipeline pieces per call (RX_P_PIPELINE)
+  bool pieces_set = false;          // chosen by the caller: else at most `pieces` (auto_pieces)
   cudaStream_t sub[3] = {nullptr, nullptr, nullptr};   // CDC, equaliser, BPS streams
   cudaEvent_t ev_fork = nullptr;
   cudaEvent_t ev_piece[3][kMaxPieces] = {};
@@ -317,6 +318,18 @@ unsigned char *u_at(rx_stream *rx, int b, int p, int64_t n) {
 }
 
 // Region layout: region 0 = [0, A), region r >= 1 = [A + (r-1) span, A + r span).
+// Pieces of a call of n waves when the caller names none.  A piece hides what comes before
+// and after it (the first piece's CDC and the last one's BPS stay in the open: about
+// 4.7 us per wave of the piece) and costs the equaliser's start and drain, about 20 us of a
+// launch: the sum is least near sqrt(n) / 2 pieces, and pieces also wait on their CDC
+// beside the equaliser, which moves the measured minimum to sqrt(n) / 3 (10 GBd QPSK, 512
+// waves: 1, 3, 6, 12, 20 pieces 10.47, 9.35, 9.23, 9.43, 9.47 ms; 32 GBd 16QAM, 31 waves:
+// 1, 2, 4, 12 pieces 1082, 1033, 1040, 1190 us; 21 waves: 1, 2, 4, 12 pieces 802, 775, 796,
+// 930 us; calls of 9 waves: 1, 2, 12 pieces 1636, 1789, 2043 us).
+int auto_pieces(const rx_stream *rx, int64_t n) {
+  return (int)std::min<double>(rx->pieces, std::max(1.0, floor(sqrt((double)n) / 3.0 + 0.5)));
+}
+
 // Symbols per BPS chunk (one warp each).  A chunk's pass is one chain of 32-symbol blocks
 // after a first block that fills its window, so with few chunks the launch lasts as long
 // as one of them: the chunk shrinks (by whole powers of two of C, so that regions still
@@ -424,7 +437,7 @@ rx_status rx_set_param(rx_stream *rx, int key, double v) {
     case RX_P_EQ_OUT: rx->eq_out = v != 0; return RX_OK;
     case RX_P_CDC_OUT: rx->cdc_out = v != 0; return RX_OK;
     case RX_P_PROFILE: rx->profile = v != 0; return RX_OK;
-    case RX_P_PIPELINE: s = as_int(1, kMaxPieces, &t); if (s == RX_OK) rx->pieces = (int)t; return s;
+    case RX_P_PIPELINE: s = as_int(1, kMaxPieces, &t); if (s == RX_OK) { rx->pieces = (int)t; rx->pieces_set = true; } return s;
     case RX_P_PRECISION: s = as_int(0, 2, &t); if (s == RX_OK) rx->fmt = (int)t; break;
     case RX_P_INNER_TRACE: s = as_int(0, (int64_t)1 << 32, &rx->inner_cap); break;
     case RX_P_WAIT_LIMIT_US:
@@ -725,7 +738,7 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
   // behind the equaliser on the SMs the equaliser leaves free.
   const int64_t n_waves = eq_work ? wave_last - wave_first : 0;
   int np = 1;
-  if (n_waves > 0) np = (int)std::min<int64_t>(std::max(1, rx->pieces), n_waves);
+  if (n_waves > 0) np = (int)std::min<int64_t>(std::max(1, rx->pieces_set ? rx->pieces : auto_pieces(rx, n_waves)), n_waves);
   np = std::min(np, kMaxPieces);
   RX_CUDA(cudaEventRecord(rx->ev_fork, st), "fork");
   for (int i = 0; i < 3; ++i) RX_CUDA(cudaStreamWaitEvent(rx->sub[i], rx->ev_fork, 0), "fork");
