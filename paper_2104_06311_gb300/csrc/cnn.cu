@@ -759,6 +759,243 @@ __global__ void pack_tc_kernel(const float *__restrict__ W, int ci_true, int co_
   }
 }
 
+// ---------------------------------------------------------------- weight gradients on tcgen05
+// All layers' weight and bias gradients in one launch, symbols as the reduction dimension
+// (K = 16 symbols per MMA): both operands are read MN-major from the row tiles as they lie
+// in memory ([n][64 channels], 128-byte swizzle), no transposition.
+//
+// Hidden layers: dW[k][ci][co] = sum_n in[n + k - 7][ci] dz[n][co].  An MMA of M = 128 rows
+// takes two taps at once: the second 64 rows are the same input rows one symbol on, which
+// is a leading offset of one row (128 bytes).  A CTA works through a chunk of tiles for two
+// pairs of taps, D in 128 columns of tensor memory; the last pair's second half (tap 15,
+// not a tap) reads a block of ones instead: db.
+//
+// Edge layers: D[4 t + f][o] = sum_n feat[n + t - 7][f] rows[n][o], with feat the input
+// features and rows = dz for the first layer (dW[t][f][o] = D), feat = dJ/dy and rows = the
+// last hidden layer's output for the last one (dW[14 - t][o][f] = D).  The features lie
+// in shared memory as pairs (x[m], x[m+1]) of 16 bytes: a core matrix (8 of M = 2 taps, 8
+// symbols) is 8 successive pairs, the next two taps are two pairs on.
+//
+// A CTA adds its part to the FP32 gradient with 16-byte atomics at the end.
+constexpr int DW_STAGES = 2;
+constexpr int DW_PAIRS = 2;                          // tap pairs per CTA of a hidden layer
+constexpr int DW_GROUPS = (KS + 1) / (2 * DW_PAIRS); // CTAs per chunk
+constexpr int DW_Z_BYTES = TC_M * 128;
+constexpr int DW_STAGE_BYTES = TC_A_BYTES + DW_Z_BYTES;
+constexpr int DW_Y_ROWS = TC_M + 32;                 // pairs that an edge tile's operand spans (rows past tap 14: unused)
+constexpr int DW_OFF_ONES = DW_STAGES * DW_STAGE_BYTES;
+constexpr int DW_ONES_BYTES = 2304;                  // 16 x 128 bytes and one more row group (core matrices 128 apart)
+constexpr int DW_OFF_Y = DW_OFF_ONES + DW_ONES_BYTES;
+constexpr int DW_OFF_BAR = DW_OFF_Y + DW_Y_ROWS * 16;
+constexpr int DW_SMEM = DW_OFF_BAR + 64 + 1024;
+constexpr unsigned DW_TMEM_COLS = 128;
+// MN-major A and B (bits 15, 16)
+constexpr unsigned DW_IDESC = TC_IDESC | (1u << 15) | (1u << 16);
+constexpr int DW_MAX_LAYERS = 8;
+
+struct DwTcLayer {
+  CUtensorMap x, z;          // hidden: input rows (142-row boxes), dz rows (128); edges: rows in z
+  const float2 *sym;         // first layer: the received symbols
+  int64_t sym_stride;
+  const bf16 *feat;          // last layer: dJ/dy rows of FEATP
+  float *dw, *db;
+  int first_block;           // of this layer in the grid
+  int chunk_tiles;
+};
+struct DwTcArgs {
+  DwTcLayer l[DW_MAX_LAYERS];
+  int L;
+  int64_t K;
+};
+
+__device__ __forceinline__ void dw_mma(unsigned d, unsigned long long a, unsigned long long b, bool acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+      :: "r"(d), "l"(a), "l"(b), "r"(DW_IDESC), "r"(acc ? 1u : 0u)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(TC_M) dw_tc_kernel(const __grid_constant__ DwTcArgs a, int *__restrict__ err) {
+  extern __shared__ unsigned char tc_raw[];
+  unsigned char *const sm = tc_raw + ((1024u - (smem_u32(tc_raw) & 1023u)) & 1023u);
+  unsigned long long *const bars = reinterpret_cast<unsigned long long *>(sm + DW_OFF_BAR);
+  unsigned *const tmem_slot = reinterpret_cast<unsigned *>(bars + 5);
+  volatile int *const fail = reinterpret_cast<volatile int *>(bars + 6);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  auto bar_full = [&](int s) { return smem_u32(&bars[s]); };
+  auto bar_free = [&](int s) { return smem_u32(&bars[DW_STAGES + s]); };
+  const unsigned bar_done = smem_u32(&bars[2 * DW_STAGES]);
+  if (warp == 0) tc_alloc(smem_u32(tmem_slot), DW_TMEM_COLS);
+  if (tid == 0) {
+    for (int i = 0; i < 2 * DW_STAGES + 1; ++i) tc_bar_init(smem_u32(&bars[i]), 1u);
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    *fail = 0;
+  }
+  for (int i = tid; i < DW_ONES_BYTES / 16; i += TC_M)
+    *reinterpret_cast<uint4 *>(sm + DW_OFF_ONES + i * 16) = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = *tmem_slot;
+  const long long deadline = tc_now() + kTcWaitNs;
+  int li = 0;
+  while (li + 1 < a.L && (int)blockIdx.x >= a.l[li + 1].first_block) ++li;
+  const DwTcLayer &y = a.l[li];
+  const bool first = li == 0, last = li == a.L - 1, edge = first || last;
+  const int rel = (int)blockIdx.x - y.first_block;
+  const int group = edge ? 0 : rel % DW_GROUPS;
+  const int64_t n_tiles = (a.K + TC_M - 1) / TC_M;
+  const int64_t t0 = (int64_t)(edge ? rel : rel / DW_GROUPS) * y.chunk_tiles;
+  const int nt = (int)min((int64_t)y.chunk_tiles, n_tiles - t0);   // >= 1
+  tc_grid_wait();
+  if (tid == 0) tc_grid_trigger();
+  auto load = [&](int i) {                            // tile i of this CTA into its stage
+    const int s = i % DW_STAGES;
+    const unsigned st = smem_u32(sm + s * DW_STAGE_BYTES);
+    const int64_t n0 = (t0 + i) * TC_M;
+    tc_expect(bar_full(s), (unsigned)((edge ? 0 : TC_A_TX) + DW_Z_BYTES));
+    if (!edge) tc_load_box(&y.x, st, n0 - HALF, bar_full(s));
+    tc_load_box(&y.z, st + TC_A_BYTES, n0, bar_full(s));
+  };
+  if (tid == 0)
+    for (int i = 0; i < min(nt, DW_STAGES); ++i) load(i);
+  const unsigned ones = smem_u32(sm + DW_OFF_ONES);
+  float4 dbp = make_float4(0.f, 0.f, 0.f, 0.f);       // last layer: this thread's part of db
+  bool ok = true;
+  int it = 0;
+  for (; it < nt; ++it) {
+    if (!edge && !ok) break;                          // thread 0 alone waits: the others come to the last wait
+    const int s = it % DW_STAGES;
+    const unsigned st = smem_u32(sm + s * DW_STAGE_BYTES);
+    if (edge) {
+      // the pairs of this tile (the MMAs of the last one are done: every thread waited below)
+      uint2 *const ysm = reinterpret_cast<uint2 *>(sm + DW_OFF_Y);
+      const int64_t n0 = (t0 + it) * TC_M;
+      for (int m = tid; m <= DW_Y_ROWS; m += TC_M) {
+        const int64_t n = n0 - HALF + m;
+        uint2 v = make_uint2(0u, 0u);
+        if (m < TC_ROWS && n >= 0 && n < a.K) {
+          if (first) {
+            const float2 p0 = __ldg(&y.sym[n]), p1 = __ldg(&y.sym[y.sym_stride + n]);
+            const __nv_bfloat162 v0 = __floats2bfloat162_rn(p0.x, p0.y), v1 = __floats2bfloat162_rn(p1.x, p1.y);
+            v = make_uint2(*reinterpret_cast<const unsigned *>(&v0), *reinterpret_cast<const unsigned *>(&v1));
+          } else {
+            v = __ldg(reinterpret_cast<const uint2 *>(y.feat + n * FEATP));
+            if (m >= HALF && m < HALF + TC_M) {       // a symbol of this tile
+              const __nv_bfloat162 v0 = *reinterpret_cast<const __nv_bfloat162 *>(&v.x);
+              const __nv_bfloat162 v1 = *reinterpret_cast<const __nv_bfloat162 *>(&v.y);
+              dbp.x += __bfloat162float(v0.x);
+              dbp.y += __bfloat162float(v0.y);
+              dbp.z += __bfloat162float(v1.x);
+              dbp.w += __bfloat162float(v1.y);
+            }
+          }
+        }
+        if (m < DW_Y_ROWS) ysm[2 * m] = v;
+        if (m > 0) ysm[2 * m - 1] = v;
+      }
+      asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+      if (__syncthreads_or(!ok)) break;
+    }
+    if (tid == 0) {
+      ok = tc_wait(bar_full(s), (unsigned)((it / DW_STAGES) & 1), deadline, fail);
+      if (ok) {
+        tc_fence_after();
+        const unsigned long long zd = tc_desc(st + TC_A_BYTES, 16u, 1024u) | (2ull << 61);
+        if (edge) {
+          // pairs: two taps on = 32 bytes along M, 8 symbols on = 128 bytes along K
+          const unsigned long long yd = tc_desc(smem_u32(sm + DW_OFF_Y), 128u, 32u);
+          const unsigned long long od = tc_desc(ones, 128u, 128u);
+#pragma unroll
+          for (int q = 0; q < TC_M / 16; ++q) {
+            dw_mma(tmem, yd + q * 16, zd + q * 128, (it | q) != 0);
+            if (first) dw_mma(tmem + 64, od, zd + q * 128, (it | q) != 0);
+          }
+        } else {
+#pragma unroll
+          for (int pr = 0; pr < DW_PAIRS; ++pr) {
+            const unsigned row = st + (unsigned)(2 * (group * DW_PAIRS + pr)) * 128u;
+            const bool db = group * DW_PAIRS + pr == (KS - 1) / 2;      // tap 14 and the ones
+            const unsigned long long xd = tc_desc(row, db ? ones - row : 128u, 1024u) | (2ull << 61);
+            const unsigned long long adv = db ? 128ull - (128ull << 16) : 128ull;   // 16 rows on; the ones stay
+#pragma unroll
+            for (int q = 0; q < TC_M / 16; ++q) dw_mma(tmem + 64 * pr, xd + q * adv, zd + q * 128, (it | q) != 0);
+          }
+        }
+        tc_commit(bar_free(s));
+      }
+    }
+    // the stage is refilled, and the pairs rewritten, once the MMAs are done
+    if (edge || it + DW_STAGES < nt) {
+      if (edge || tid == 0) {
+        if (ok) ok = tc_wait(bar_free(s), (unsigned)((it / DW_STAGES) & 1), deadline, fail);
+        if (ok && tid == 0 && it + DW_STAGES < nt) load(it + DW_STAGES);
+      }
+    }
+  }
+  if (tid == 0 && ok) tc_commit(bar_done);            // every MMA
+  if (ok) ok = tc_wait(bar_done, 0u, deadline, fail);
+  if (*fail && tid == 0) {
+    for (int i = max(0, it - 1); i < min(nt, it + DW_STAGES); ++i) tc_drain(bar_full(i % DW_STAGES), (unsigned)((i / DW_STAGES) & 1));
+  }
+  tc_fence_after();
+  if (!__syncthreads_or(!ok)) {
+    const unsigned ta = tmem + ((unsigned)(warp * 32) << 16);
+    const int r = tid;                                // accumulator row
+#pragma unroll 1
+    for (int h = 0; h < 4; ++h) {                     // 32 columns at a time
+      float v[32];
+      tc_ld32(ta + 32 * h, v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+      const int c0 = (h & 1) * 32;
+      float *dst = nullptr;
+      if (!edge) {
+        const int pr = group * DW_PAIRS + (h >> 1), k = 2 * pr + (r >> 6), ci = r & 63;
+        if (k < KS) dst = y.dw + ((size_t)k * CH + ci) * CH + c0;
+        else if (ci == 0) dst = y.db + c0;
+      } else if (first) {
+        if (h < 2 && r < KS * FEAT) dst = y.dw + (size_t)r * CH + c0;
+        else if (h >= 2 && r == 0) dst = y.db + c0;
+      }
+      if (dst) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          atomicAdd(reinterpret_cast<float4 *>(dst) + q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+      }
+      if (last && h < 2) {
+        // dW[14 - t][o][f] of row 4 t + f: four lanes hold the four f of one t
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+          const float v1 = __shfl_down_sync(0xffffffffu, v[q], 1), v2 = __shfl_down_sync(0xffffffffu, v[q], 2),
+                      v3 = __shfl_down_sync(0xffffffffu, v[q], 3);
+          if (r < KS * FEAT && (lane & 3) == 0)
+            atomicAdd(reinterpret_cast<float4 *>(y.dw + ((size_t)(KS - 1 - (r >> 2)) * CH + c0 + q) * FEAT),
+                      make_float4(v[q], v1, v2, v3));
+        }
+      }
+    }
+    if (last) {
+      for (int o = 16; o >= 1; o >>= 1) {
+        dbp.x += __shfl_xor_sync(0xffffffffu, dbp.x, o);
+        dbp.y += __shfl_xor_sync(0xffffffffu, dbp.y, o);
+        dbp.z += __shfl_xor_sync(0xffffffffu, dbp.z, o);
+        dbp.w += __shfl_xor_sync(0xffffffffu, dbp.w, o);
+      }
+      if (lane == 0) atomicAdd(reinterpret_cast<float4 *>(y.db), dbp);
+    }
+  } else if (tid == 0) {
+    atomicExch(err, 1);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_fence_after();
+    tc_dealloc(tmem, DW_TMEM_COLS);
+  }
+}
+
 struct DwArgs {
   const bf16 *in;     // layer input [K][CIN]
   const bf16 *dz;     // dJ/d(pre-activation) [K][COUT]
@@ -982,10 +1219,13 @@ struct rx_cnn {
   std::vector<bf16 *> wf, wb;
   std::vector<bf16 *> wtc_f, wtc_b;    // tcgen05 operand images (wtc_b: none for the first layer)
   bool use_tc = true;
-  int *err = nullptr;                  // sticky device error word (bounded waits)
-  bf16 *x0 = nullptr, *dout = nullptr, *dza = nullptr, *dzb = nullptr;
+  int *err = nullptr;                  // sticky device error word (bounded waits), in res
+  bf16 *x0 = nullptr, *dout = nullptr;
+  std::vector<bf16 *> dz;              // dJ/d(pre-activation) of layers 0 .. L-2
   std::vector<bf16 *> h;               // hidden outputs h_1 .. h_{L-1}
-  double *loss = nullptr;
+  struct Result { double loss; int err, pad; };
+  Result *res = nullptr, *h_res = nullptr;   // device, and the pinned copy that grads reads back
+  double *loss = nullptr;              // in res
   int64_t step = 0;
   std::vector<void *> allocs;
   std::string msg;
@@ -1024,6 +1264,8 @@ rx_status calloc_dev(rx_cnn *c, Tp **p, size_t count) {
 }
 
 void release(rx_cnn *c) {
+  if (c->h_res) cudaFreeHost(c->h_res);
+  c->h_res = nullptr;
   for (void *p : c->allocs) cudaFree(p);
   c->allocs.clear();
 }
@@ -1131,12 +1373,12 @@ cudaError_t launch_conv_tc(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool p
 }
 
 template <bool SRC_Z, int EPI>
-cudaError_t launch_edge_in(rx_cnn *c, const ConvArgs &a, const bf16 *img) {
+cudaError_t launch_edge_in(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool pdl) {
   KTimer tm(c, EPI == EPI_MASK ? RX_CNN_K_DX : RX_CNN_K_FWD_EDGE);
   CUtensorMap tout;
   const cudaError_t e = row_map(&tout, a.out, a.K, 32);
   if (e != cudaSuccess) return e;
-  return launch_tc(edge_in_kernel<SRC_Z, EPI>, tc_grid(c, a.K, TC_M, 6), TC_M, 0, c->stream, false, tout, a,
+  return launch_tc(edge_in_kernel<SRC_Z, EPI>, tc_grid(c, a.K, TC_M, 6), TC_M, 0, c->stream, pdl, tout, a,
                    (const void *)img, c->err);
 }
 
@@ -1150,7 +1392,7 @@ cudaError_t launch_edge_out(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool 
 }
 
 template <int CIN, int COUT>
-cudaError_t launch_dw(rx_cnn *c, const bf16 *in, const bf16 *dz, int64_t K, int l) {
+cudaError_t launch_dw(rx_cnn *c, const bf16 *in, const bf16 *dz, int64_t K, int l, float *G) {
   KTimer tm(c, RX_CNN_K_DW);
   DwArgs a;
   a.in = in;
@@ -1160,8 +1402,8 @@ cudaError_t launch_dw(rx_cnn *c, const bf16 *in, const bf16 *dz, int64_t K, int 
   // longer CTAs (their tile copies double-buffered) beat more, shorter ones
   const int64_t want = std::max<int64_t>(1, (int64_t)c->sms / (KS / TG));
   a.chunk = ((K + want - 1) / want + TM - 1) / TM * TM;
-  a.dw = c->G + c->off_w[l];
-  a.db = c->G + c->off_b[l];
+  a.dw = G + c->off_w[l];
+  a.db = G + c->off_b[l];
   a.ci_true = c->ci[l];
   a.co_true = c->co[l];
   dim3 grid((unsigned)((K + a.chunk - 1) / a.chunk), KS / TG);
@@ -1169,6 +1411,38 @@ cudaError_t launch_dw(rx_cnn *c, const bf16 *in, const bf16 *dz, int64_t K, int 
   cudaFuncSetAttribute(dw_kernel<CIN, COUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   dw_kernel<CIN, COUT><<<grid, kThreads, smem, c->stream>>>(a);
   return cudaGetLastError();
+}
+
+// Every layer's gradients into G (zeroed before the forward pass) from the stored rows.
+cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, float *G) {
+  KTimer tm(c, RX_CNN_K_DW);
+  DwTcArgs a;
+  memset(&a, 0, sizeof(a));
+  a.L = c->L;
+  a.K = K;
+  const int64_t n_tiles = (K + TC_M - 1) / TC_M;
+  // one wave of at most three CTAs per SM: two per SM over the hidden layers, a half over each
+  // edge layer
+  const int64_t want_h = std::max<int64_t>(1, 2 * c->sms / (DW_GROUPS * std::max(1, c->L - 2)));
+  const int64_t want_e = std::max(1, c->sms / 2);
+  int blocks = 0;
+  for (int l = 0; l < c->L; ++l) {
+    DwTcLayer &y = a.l[l];
+    const bool edge = l == 0 || l == c->L - 1;
+    const int64_t chunk = (n_tiles + (edge ? want_e : want_h) - 1) / (edge ? want_e : want_h);
+    y.chunk_tiles = (int)chunk;
+    y.first_block = blocks;
+    blocks += (int)((n_tiles + chunk - 1) / chunk) * (edge ? 1 : DW_GROUPS);
+    y.dw = G + c->off_w[l];
+    y.db = G + c->off_b[l];
+    y.sym = z;
+    y.sym_stride = zs;
+    y.feat = c->dout;
+    cudaError_t e = row_map(&y.z, l == c->L - 1 ? c->h[l - 1] : c->dz[l], K, TC_M);
+    if (e == cudaSuccess && !edge) e = row_map(&y.x, c->h[l - 1], K, TC_ROWS);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_tc(dw_tc_kernel, blocks, TC_M, DW_SMEM, c->stream, true, a, c->err);
 }
 
 rx_status check_sym(rx_cnn *c, const float *p, int64_t stride, int64_t K, const char *what) {
@@ -1180,7 +1454,7 @@ rx_status check_sym(rx_cnn *c, const float *p, int64_t stride, int64_t K, const 
 
 // Forward pass; with t, also the loss and dJ/dy.  y may be NULL.
 rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, const float *t, int64_t ts, int64_t K) {
-  if (t || !c->use_tc) {   // the feature rows: the weight gradient's input, and the mma.sync path's
+  if (!c->use_tc) {
     const int g = (int)std::min<int64_t>((K + 255) / 256, 4 * c->sms);
     features_kernel<<<std::max(1, g), 256, 0, c->stream>>>(reinterpret_cast<const float2 *>(z), zs, K, c->x0);
     CX_CUDA(cudaGetLastError(), "features");
@@ -1199,7 +1473,7 @@ rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, c
       a.in = l == 0 ? c->x0 : c->h[l - 1];
       a.out = c->h[l];
       if (l == 0 && c->use_tc) {
-        CX_CUDA((launch_edge_in<true, EPI_RELU>(c, a, c->wtc_f[l])), "conv (first)");
+        CX_CUDA((launch_edge_in<true, EPI_RELU>(c, a, c->wtc_f[l], false)), "conv (first)");
       } else if (l == 0) {
         CX_CUDA((launch_conv<FEATP, CH, EPI_RELU>(c, a)), "conv");
       } else if (c->use_tc) {
@@ -1223,21 +1497,21 @@ rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, c
   return RX_OK;
 }
 
-// Backward pass into c->G (zeroed here) from c->dout and the stored activations.
-rx_status backward(rx_cnn *c, int64_t K) {
-  CX_CUDA(cudaMemsetAsync(c->G, 0, (size_t)c->n_params * sizeof(float), c->stream), "zero grads");
+// Backward pass into G (zeroed before the forward pass) from c->dout and the stored
+// activations; z: the forward pass's input.
+rx_status backward(rx_cnn *c, const float *z, int64_t zs, int64_t K, float *G) {
   const int L = c->L;
-  const bf16 *dz = c->dout;      // [K][16] for the last layer
-  bf16 *bufs[2] = {c->dza, c->dzb};
   for (int l = L - 1; l >= 0; --l) {
-    const bf16 *in = l == 0 ? c->x0 : c->h[l - 1];
     const bool last = l == L - 1;
-    if (l == 0) {
-      CX_CUDA((launch_dw<FEATP, CH>(c, in, dz, K, l)), "weight gradient");
-    } else if (last) {
-      CX_CUDA((launch_dw<CH, FEATP>(c, in, dz, K, l)), "weight gradient");
-    } else {
-      CX_CUDA((launch_dw<CH, CH>(c, in, dz, K, l)), "weight gradient");
+    const bf16 *dz = last ? c->dout : c->dz[l];      // [K][16] for the last layer
+    if (!c->use_tc) {
+      if (l == 0) {
+        CX_CUDA((launch_dw<FEATP, CH>(c, c->x0, dz, K, l, G)), "weight gradient");
+      } else if (last) {
+        CX_CUDA((launch_dw<CH, FEATP>(c, c->h[l - 1], dz, K, l, G)), "weight gradient");
+      } else {
+        CX_CUDA((launch_dw<CH, CH>(c, c->h[l - 1], dz, K, l, G)), "weight gradient");
+      }
     }
     if (l == 0) break;
     // dJ/d(pre-activation of layer l - 1) = (dz conv W_l^T reversed) * [h_{l-1} > 0]
@@ -1247,19 +1521,18 @@ rx_status backward(rx_cnn *c, int64_t K) {
     a.K = K;
     a.w = c->wb[l];
     a.mask = c->h[l - 1];
-    bf16 *out = bufs[l & 1];
-    a.out = out;
+    a.out = c->dz[l - 1];
     if (last && c->use_tc) {
-      CX_CUDA((launch_edge_in<false, EPI_MASK>(c, a, c->wtc_b[l])), "input gradient");
+      CX_CUDA((launch_edge_in<false, EPI_MASK>(c, a, c->wtc_b[l], true)), "input gradient");
     } else if (last) {
       CX_CUDA((launch_conv<FEATP, CH, EPI_MASK>(c, a)), "input gradient");
     } else if (c->use_tc) {
-      CX_CUDA(launch_conv_tc<EPI_MASK>(c, a, c->wtc_b[l], false), "input gradient (tensor memory)");
+      CX_CUDA(launch_conv_tc<EPI_MASK>(c, a, c->wtc_b[l], true), "input gradient (tensor memory)");
     } else {
       CX_CUDA((launch_conv<CH, CH, EPI_MASK>(c, a)), "input gradient");
     }
-    dz = out;
   }
+  if (c->use_tc) CX_CUDA(launch_dw_tc(c, reinterpret_cast<const float2 *>(z), zs, K, G), "weight gradients");
   return RX_OK;
 }
 
@@ -1307,6 +1580,7 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   if (e == cudaSuccess) e = conv_prepare<CH, CH, EPI_MASK>();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_kernel<EPI_RELU>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(conv_tc_kernel<EPI_MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(dw_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DW_SMEM);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(edge_out_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, ED_OUT_SMEM);
   if (e != cudaSuccess) {
     delete c;
@@ -1326,7 +1600,6 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   c->wb.assign(layers, nullptr);
   c->wtc_f.assign(layers, nullptr);
   c->wtc_b.assign(layers, nullptr);
-  CX_ALLOC(c->err, 1);
   for (int l = 0; l < layers; ++l) {
     const size_t n = l == 0 || l == layers - 1 ? (size_t)KS * CH * 8 : (size_t)KS * CH * CH;   // edges: at most
     CX_ALLOC(c->wtc_f[l], n);
@@ -1340,17 +1613,24 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   const size_t K = (size_t)max_symbols;
   CX_ALLOC(c->x0, K * FEATP);
   CX_ALLOC(c->dout, K * FEATP);
-  CX_ALLOC(c->dza, K * CH);
-  CX_ALLOC(c->dzb, K * CH);
+  c->dz.assign(layers - 1, nullptr);
+  for (int l = 0; l < layers - 1; ++l) CX_ALLOC(c->dz[l], K * CH);
   c->h.assign(layers - 1, nullptr);
   for (int l = 0; l < layers - 1; ++l) CX_ALLOC(c->h[l], K * CH);
-  CX_ALLOC(c->loss, 1);
+  CX_ALLOC(c->res, 1);
+  c->loss = &c->res->loss;
+  c->err = &c->res->err;
+  if (cudaMallocHost((void **)&c->h_res, sizeof(rx_cnn::Result)) != cudaSuccess) {
+    cudaGetLastError();
+    release(c);
+    return cfail(c, RX_ENOMEM, "pinned result");
+  }
 #undef CX_ALLOC
   CX_CUDA(cudaMemset(c->P, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->M, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->V, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->dout, 0, K * FEATP * sizeof(bf16)), "init");   // channels 4..15 stay zero
-  CX_CUDA(cudaMemset(c->err, 0, sizeof(int)), "init");
+  CX_CUDA(cudaMemset(c->res, 0, sizeof(rx_cnn::Result)), "init");
   for (int l : {0, layers - 1}) {        // padding of the edge layers' images
     CX_CUDA(cudaMemset(c->wtc_f[l], 0, (size_t)KS * CH * 8 * sizeof(bf16)), "init");
     if (c->wtc_b[l]) CX_CUDA(cudaMemset(c->wtc_b[l], 0, (size_t)KS * CH * 8 * sizeof(bf16)), "init");
@@ -1376,12 +1656,21 @@ rx_status rx_cnn_set_params(rx_cnn *c, const float *params) {
 }
 
 namespace {
+rx_status timed_out(rx_cnn *c) { return cfail(c, RX_ETIMEOUT, "a bounded device wait gave up (tensor-core convolution)"); }
+
+// Forward and backward pass: the loss in c->res, the gradients in G.
+rx_status gradients(rx_cnn *c, const float *z, int64_t zs, const float *t, int64_t ts, int64_t K, float *G) {
+  CX_CUDA(cudaMemsetAsync(c->loss, 0, sizeof(double), c->stream), "loss");
+  CX_CUDA(cudaMemsetAsync(G, 0, (size_t)c->n_params * sizeof(float), c->stream), "zero grads");
+  const rx_status s = forward(c, z, zs, nullptr, 0, t, ts, K);
+  return s == RX_OK ? backward(c, z, zs, K, G) : s;
+}
+
 rx_status check_err(rx_cnn *c) {
   int h = 0;
   CX_CUDA(cudaMemcpyAsync(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost, c->stream), "error word");
   CX_CUDA(cudaStreamSynchronize(c->stream), "error word");
-  if (h) return cfail(c, RX_ETIMEOUT, "a bounded device wait gave up (tensor-core convolution)");
-  return RX_OK;
+  return h ? timed_out(c) : RX_OK;
 }
 }  // namespace
 
@@ -1422,15 +1711,16 @@ rx_status rx_cnn_grads(rx_cnn *c, const float *z, int64_t zs, const float *t, in
   rx_status s = check_sym(c, z, zs, K, "input");
   if (s == RX_OK) s = check_sym(c, t, ts, K, "target");
   if (s != RX_OK) return s;
-  CX_CUDA(cudaMemsetAsync(c->loss, 0, sizeof(double), c->stream), "loss");
-  s = forward(c, z, zs, nullptr, 0, t, ts, K);
-  if (s == RX_OK) s = backward(c, K);
+  // straight into the caller's buffer where it takes the kernels' 16-byte atomics
+  float *G = (uintptr_t)grads_dev % 16 == 0 ? grads_dev : c->G;
+  s = gradients(c, z, zs, t, ts, K, G);
   if (s != RX_OK) return s;
-  CX_CUDA(cudaMemcpyAsync(grads_dev, c->G, (size_t)c->n_params * sizeof(float), cudaMemcpyDeviceToDevice, c->stream),
-          "grads");
-  CX_CUDA(cudaMemcpyAsync(loss, c->loss, sizeof(double), cudaMemcpyDeviceToHost, c->stream), "loss");
+  if (G != grads_dev)
+    CX_CUDA(cudaMemcpyAsync(grads_dev, G, (size_t)c->n_params * sizeof(float), cudaMemcpyDeviceToDevice, c->stream), "grads");
+  CX_CUDA(cudaMemcpyAsync(c->h_res, c->res, sizeof(rx_cnn::Result), cudaMemcpyDeviceToHost, c->stream), "loss");
   CX_CUDA(cudaStreamSynchronize(c->stream), "grads");
-  return check_err(c);
+  *loss = c->h_res->loss;
+  return c->h_res->err ? timed_out(c) : RX_OK;
 }
 
 rx_status rx_cnn_train_step(rx_cnn *c, const float *z, int64_t zs, const float *t, int64_t ts, int64_t K, float lr,
@@ -1441,9 +1731,7 @@ rx_status rx_cnn_train_step(rx_cnn *c, const float *z, int64_t zs, const float *
   rx_status s = check_sym(c, z, zs, K, "input");
   if (s == RX_OK) s = check_sym(c, t, ts, K, "target");
   if (s != RX_OK) return s;
-  CX_CUDA(cudaMemsetAsync(c->loss, 0, sizeof(double), c->stream), "loss");
-  s = forward(c, z, zs, nullptr, 0, t, ts, K);
-  if (s == RX_OK) s = backward(c, K);
+  s = gradients(c, z, zs, t, ts, K, c->G);
   if (s != RX_OK) return s;
   c->step += 1;
   const float c1 = (float)(1.0 - pow(0.9, (double)c->step));
