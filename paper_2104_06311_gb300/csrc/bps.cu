@@ -160,16 +160,15 @@ constexpr int kBlkNb = 16;
 // a block is at a constant offset.
 __host__ __device__ inline int pass1_blk_ys_cap(int chunk, int Nb) { return chunk + 2 * Nb + 32; }
 __host__ __device__ inline size_t pass1_blk_warp_bytes(int chunk, int Nb) {
-  return (size_t)pass1_blk_ys_cap(chunk, Nb) * sizeof(float2) + (size_t)((chunk + 15) / 16) * 16;
+  return (size_t)pass1_blk_ys_cap(chunk, Nb) * sizeof(float2) + (size_t)((chunk + 15) / 16) * 16 + 32 * sizeof(unsigned);
 }
 
 template <int MB, bool NEED_S2, bool EDGE, int M>
 __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_hi, float2 rot, int nt, int lane,
-                                             int8_t *bq, int &R, float &s2) {
+                                             int8_t *bq, unsigned *ties, int &R, float &s2) {
   constexpr unsigned FULL = 0xffffffffu;
-  // distance of staged position m at this lane's angle (zero outside the stream)
-  auto dd = [&](const float2 *yb, int off, int m) -> float {
-    const float2 w = cmul(yb[off], rot);
+  auto dist = [](float2 v, float2 ph) -> float {
+    const float2 w = cmul(v, ph);
     float ex, ey;
     if (MB == 2) {
       ex = fabsf(w.x) - 0.70710678118654752f;
@@ -178,7 +177,11 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
       ex = fabsf(fabsf(w.x) - 2.f) - 1.f;
       ey = fabsf(fabsf(w.y) - 2.f) - 1.f;
     }
-    const float d = ex * ex + ey * ey;
+    return ex * ex + ey * ey;
+  };
+  // distance of staged position m at this lane's angle (zero outside the stream)
+  auto dd = [&](const float2 *yb, int off, int m) -> float {
+    const float d = dist(yb[off], rot);
     return (EDGE && (m < v_lo || m >= v_hi)) ? 0.f : d;
   };
   float d0[32], d1[32];
@@ -188,9 +191,9 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
   if constexpr (M > 1) {
 #pragma unroll
     for (int r = 1; r < M; ++r) {
-      float t = 0.f;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) t += dd(ys, 32 * r + j, 32 * r + j);
+      float t = 0.f;                              // rolled: the instruction cache holds the main loop
+#pragma unroll 4
+      for (int j = 0; j < 32; ++j) t += dd(ys + 32 * r, j, 32 * r + j);
       T[r - 1] = t;
     }
   }
@@ -214,21 +217,22 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
       for (int r = 0; r < M - 1; ++r) mid += T[r];
     }
     float pre = 0.f;
-    int mybs = 0;                                 // lane i: bhat of symbol base + i
+    __syncwarp();                                 // the last block's ties are read
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       pre += d1[i];
-      const unsigned key = __float_as_uint((d0[i] + mid) + pre);   // D >= 0: float order = bit order
+      const float D = M > 1 ? (d0[i] + mid) + pre : d0[i] + pre;
+      const unsigned key = __float_as_uint(D);   // D >= 0: float order = bit order
       const unsigned mn = __reduce_min_sync(FULL, key);
-      const int bs = __ffs(__ballot_sync(FULL, key == mn)) - 1;
-      mybs = lane == i ? bs : mybs;
-      if (NEED_S2) {   // d of the symbol itself (position 32 q + i + 16 M) at angle bs
-        float own;
-        if (M == 1) own = i < 16 ? d0[i + 16] - (i + 16 < 31 ? d0[i + 17] : 0.f) : d1[i - 16];
-        else own = dd(yb, i + 16 * M, base + i + 16 * M);
-        const float add = __shfl_sync(FULL, own, bs);
-        s2 += i < cnt ? add : 0.f;
-      }
+      const unsigned tie = __ballot_sync(FULL, key == mn);
+      if (lane == 0) ties[i] = tie;               // (a store costs the busy integer pipe nothing, a select per lane two)
+    }
+    __syncwarp();
+    const int mybs = __ffs(ties[lane]) - 1;       // lane i: bhat of symbol base + i
+    if (NEED_S2) {   // d of lane i's symbol (position 32 q + i + 16 M) at its angle
+      const float2 rb = make_float2(__shfl_sync(FULL, rot.x, mybs), __shfl_sync(FULL, rot.y, mybs));
+      const float own = dist(yb[lane + 16 * M], rb);
+      s2 += lane < cnt ? own : 0.f;
     }
     // unwrap steps of the block's symbols at once (r of the chunk's first symbol: the scan)
     const int up = __shfl_up_sync(FULL, mybs, 1);
@@ -250,7 +254,11 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
       T[M - 2] = t;
     }
   }
-  if (MB == 4) s2 *= 0.1f;
+  if (NEED_S2) {
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) s2 += __shfl_xor_sync(FULL, s2, o);
+    if (MB == 4) s2 *= 0.1f;
+  }
 }
 
 template <int MB, bool NEED_S2, int M>
@@ -264,6 +272,7 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_blk(BpsLaunch L) {
   char *base = reinterpret_cast<char *>(smem_raw) + (size_t)warp * pass1_blk_warp_bytes(L.chunk, Nb);
   float2 *ys = reinterpret_cast<float2 *>(base);
   int8_t *bq = reinterpret_cast<int8_t *>(ys + pass1_blk_ys_cap(L.chunk, Nb));
+  unsigned *ties = reinterpret_cast<unsigned *>(bq + (L.chunk + 15) / 16 * 16);
   const int64_t a = chunk_lo(L, j), b = min(a + (int64_t)L.chunk, L.k_hi);
   const int64_t lo = a - Nb;                     // ys[m] holds symbol lo + m
   const int nt = (int)(b - a);
@@ -285,9 +294,9 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_blk(BpsLaunch L) {
   float s2 = 0.f;
   if (v_lo > 0 || v_hi < n_ys) {                  // the window touches a stream end
     pass1_blocks<MB, NEED_S2, true, M>(ys, (int)max(v_lo, (int64_t)0), (int)min(v_hi, (int64_t)n_ys), rot, nt, lane,
-                                       bq, R, s2);
+                                       bq, ties, R, s2);
   } else {
-    pass1_blocks<MB, NEED_S2, false, M>(ys, 0, n_ys, rot, nt, lane, bq, R, s2);
+    pass1_blocks<MB, NEED_S2, false, M>(ys, 0, n_ys, rot, nt, lane, bq, ties, R, s2);
   }
   __syncwarp();
   int8_t *bh = L.bhat + (int64_t)p * L.bh_stride - L.bh_base;
@@ -355,7 +364,8 @@ __global__ void __launch_bounds__(1024) bps_scan(BpsLaunch L) {
     for (int64_t c = q0 + lane; c < q1; c += 32) acc += (double)L.chunk_s2[(int64_t)p * n + c];
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) L.region_s2[(int64_t)p * (r_hi - r_lo) + (r - r_lo)] = acc / (double)(e_r - s_r);
+    // 1 / sigma^2, what the demapping multiplies by
+    if (lane == 0) L.region_s2[(int64_t)p * (r_hi - r_lo) + (r - r_lo)] = 1.0 / (acc / (double)(e_r - s_r));
   }
 }
 
@@ -396,16 +406,37 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_demap(BpsLaunch L) {
   const float2 *y = L.y + (int64_t)p * L.y_stride - L.y_base;
   const int8_t *bh = L.bhat + (int64_t)p * L.bh_stride - L.bh_base;
   int64_t m = L.chunk_m[(int64_t)p * L.n_chunks + j];
-  const int64_t r_lo = L.k_lo < L.A ? 0 : 1 + (L.k_lo - L.A) / L.span;
-  const int64_t r_hi = L.k_hi <= L.A ? 1 : 1 + (L.k_hi - 1 - L.A) / L.span + 1;
-  const int64_t region = a < L.A ? 0 : 1 + (a - L.A) / L.span;
-  const float s2inv = (float)(1.0 / L.region_s2[(int64_t)p * (r_hi - r_lo) + (region - r_lo)]);
+  float s2inv = 0.f;
+  if (L.llr) {
+    const int64_t r_lo = L.k_lo < L.A ? 0 : 1 + (L.k_lo - L.A) / L.span;
+    const int64_t r_hi = L.k_hi <= L.A ? 1 : 1 + (L.k_hi - 1 - L.A) / L.span + 1;
+    const int64_t region = a < L.A ? 0 : 1 + (a - L.A) / L.span;
+    s2inv = (float)L.region_s2[(int64_t)p * (r_hi - r_lo) + (region - r_lo)];
+  }
+  // symbols and angles two blocks ahead of their use: a chunk is one chain of loads otherwise
+  auto load = [&](int64_t base, float2 &yv, int &cur) {
+    const int64_t k = base + lane;
+    yv = k < b ? y[k] : make_float2(0.f, 0.f);
+    cur = k < b ? (int)bh[k] : 0;
+  };
+  float2 y0, y1;
+  int c0, c1;
+  load(a, y0, c0);
+  load(a + 32, y1, c1);
+  int before = a > 0 ? (int)bh[a - 1] : 0;       // the angle in front of the block
   for (int64_t base = a; base < b; base += 32) {
     const int64_t k = base + lane;
     const bool valid = k < b;
-    const int cur = valid ? (int)bh[k] : 0;
+    const int cur = c0;
+    const float2 yk = y0;
+    y0 = y1;
+    c0 = c1;
+    load(base + 64, y1, c1);
+    const int up = __shfl_up_sync(0xffffffffu, cur, 1);
+    const int prev = lane == 0 ? before : up;
+    before = __shfl_sync(0xffffffffu, cur, 31);
     int r = 0;
-    if (valid && k > 0) r = unwrap_step((int)bh[k - 1], cur);
+    if (valid && k > 0) r = unwrap_step(prev, cur);
     // inclusive warp scan of r
     int sc = r;
 #pragma unroll
@@ -421,7 +452,7 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_demap(BpsLaunch L) {
     unsigned v = 0;
     const int64_t jo = k - L.out_first;
     if (valid) {
-      z = cmul(y[k], make_float2(rc, rs));
+      z = cmul(yk, make_float2(rc, rs));
       switch ((int)(((mk % 4) + 4) % 4)) {  // (-j)^m
         case 1: z = make_float2(z.y, -z.x); break;
         case 2: z = make_float2(-z.x, -z.y); break;
