@@ -689,11 +689,34 @@ __global__ void copy_cols_kernel(float2 *dst, int64_t ds, const float2 *src, int
   dst[i] = src[i];
   dst[ds + i] = src[ss + i];
 }
-__global__ void copy_cols_i8_kernel(int8_t *dst, int64_t ds, const int8_t *src, int64_t ss, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  dst[i] = src[i];
-  dst[ds + i] = src[ss + i];
+// A stream's carried columns (CDC output; equaliser output and angles) to the other buffer
+// of each pair, both rows of each, in one launch: blocks below bu take u, the rest y and
+// bhat.  A few hundred kilobytes, so the launches were the cost (three took 10 us).
+template <class S>
+__global__ void __launch_bounds__(256) slide_kernel(SlideArgs a, unsigned bu) {
+  if (blockIdx.x < bu) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= a.nu) return;
+    S *d = static_cast<S *>(a.u_dst);
+    const S *s = static_cast<const S *>(a.u_src);
+    d[i] = s[i];
+    d[a.u_stride + i] = s[a.u_stride + i];
+  } else {
+    const int64_t i = (int64_t)(blockIdx.x - bu) * 256 + threadIdx.x;
+    if (i >= a.ny) return;
+    a.y_dst[i] = a.y_src[i];
+    a.y_dst[a.y_stride + i] = a.y_src[a.y_stride + i];
+    a.b_dst[i] = a.b_src[i];
+    a.b_dst[a.y_stride + i] = a.b_src[a.y_stride + i];
+  }
+}
+
+cudaError_t launch_slide(const SlideArgs &a, cudaStream_t s) {
+  const unsigned bu = (unsigned)((a.nu + 255) / 256), by = (unsigned)((a.ny + 255) / 256);
+  if (bu + by == 0) return cudaSuccess;
+  if (a.fmt == RX_FMT_F32) slide_kernel<float2><<<bu + by, 256, 0, s>>>(a, bu);
+  else slide_kernel<uint32_t><<<bu + by, 256, 0, s>>>(a, bu);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_copy_cols(float2 *dst, int64_t dst_stride, const float2 *src,
@@ -701,12 +724,6 @@ cudaError_t launch_copy_cols(float2 *dst, int64_t dst_stride, const float2 *src,
   if (n <= 0) return cudaSuccess;
   copy_cols_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dst, dst_stride, src, src_stride, n);
   return cudaGetLastError();
-}
-__global__ void copy_cols_u32_kernel(uint32_t *dst, int64_t ds, const uint32_t *src, int64_t ss, int64_t n) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  dst[i] = src[i];
-  dst[ds + i] = src[ss + i];
 }
 template <int FMT>
 __global__ void cols_to_f32_kernel(float2 *dst, int64_t ds, const void *src_v, int64_t ss, int64_t n) {
@@ -716,16 +733,6 @@ __global__ void cols_to_f32_kernel(float2 *dst, int64_t ds, const void *src_v, i
   if (i >= n) return;
   dst[i] = ld2(src[i]);
   dst[ds + i] = ld2(src[ss + i]);
-}
-
-cudaError_t launch_copy_cols_fmt(void *dst, int64_t dst_stride, const void *src, int64_t src_stride, int64_t n,
-                                 int fmt, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  if (fmt == RX_FMT_F32)
-    return launch_copy_cols((float2 *)dst, dst_stride, (const float2 *)src, src_stride, n, s);
-  copy_cols_u32_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>((uint32_t *)dst, dst_stride, (const uint32_t *)src,
-                                                                  src_stride, n);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_cols_to_f32(float2 *dst, int64_t dst_stride, const void *src, int64_t src_stride, int64_t n,
@@ -738,13 +745,6 @@ cudaError_t launch_cols_to_f32(float2 *dst, int64_t dst_stride, const void *src,
     case RX_FMT_BF16: cols_to_f32_kernel<RX_FMT_BF16><<<g, 256, 0, s>>>(dst, dst_stride, src, src_stride, n); break;
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_copy_cols_i8(int8_t *dst, int64_t dst_stride, const int8_t *src,
-                                int64_t src_stride, int64_t n, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  copy_cols_i8_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(dst, dst_stride, src, src_stride, n);
   return cudaGetLastError();
 }
 

@@ -900,6 +900,8 @@ __device__ __forceinline__ void eq_body(const EqLaunch &L, const int cta, EqSmem
   if (threadIdx.x == 0) {
     sm.ybuf[0][31] = sm.ybuf[1][31] = make_float2(0.f, 0.f);
   }
+  if (cta == 0 && L.barrier_next != nullptr)
+    for (int k = threadIdx.x; k < kEqBarrierWords; k += G::NT) L.barrier_next[k] = 0u;
   for (int m = threadIdx.x; m < 256; m += G::NT) {
     float s, c;
     sincospif((float)m / 128.f, &s, &c);

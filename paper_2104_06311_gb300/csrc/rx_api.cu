@@ -79,7 +79,8 @@ struct rx_stream {
   double *trace_fo = nullptr;
   int64_t trace_cap = 4096;
   int8_t *inner = nullptr;          // [2][inner_cap] inner BPS angles (RX_P_INNER_TRACE)
-  unsigned *barrier = nullptr;
+  unsigned *barrier = nullptr;      // two sets of kEqBarrierWords
+  bool bar_set = false;             // the set of the next equaliser launch (zero by then)
   int *err = nullptr;
   int *chunk_r = nullptr;
   float *chunk_s2 = nullptr;
@@ -236,19 +237,34 @@ int eq_grid(const rx_stream *rx) {
   return (rx->eq_alt && rx->eq_alt_ok && rx->eq_blocks == 2 * rx->P) ? 4 * rx->P : rx->eq_blocks;
 }
 
+// Start state of a stream, in one launch.
+__global__ void stream_init_kernel(EqState *st, int c, int64_t *m_carry, int *err, double *trace_fo, int64_t n_trace_fo,
+                                   int8_t *inner, int64_t n_inner, unsigned *barrier) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = i0; i < n_trace_fo; i += step) trace_fo[i] = 0.0;
+  for (int64_t i = i0; i < n_inner; i += step) inner[i] = -1;
+  for (int64_t i = i0; i < 2 * kEqBarrierWords; i += step) barrier[i] = 0u;
+  static_assert(sizeof(EqState) % sizeof(unsigned) == 0, "whole words");
+  if (blockIdx.x == 0) {
+    for (int k = threadIdx.x; k < (int)(sizeof(EqState) / sizeof(unsigned)); k += blockDim.x)
+      reinterpret_cast<unsigned *>(st)[k] = 0u;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      st->taps[0][0][c].x = st->taps[1][1][c].x = 1.f;
+      m_carry[0] = m_carry[1] = 0;
+      *err = 0;
+    }
+  }
+}
+
 rx_status init_device_state(rx_stream *rx) {
-  EqState s;
-  memset(&s, 0, sizeof(s));
-  const int c = (rx->T - 1) / 2;
-  s.taps[0][0][c] = make_float2(1.f, 0.f);
-  s.taps[1][1][c] = make_float2(1.f, 0.f);
-  RX_CUDA(cudaMemcpyAsync(rx->st, &s, sizeof(s), cudaMemcpyHostToDevice, rx->stream), "state init");
-  RX_CUDA(cudaMemsetAsync(rx->m_carry, 0, 2 * sizeof(int64_t), rx->stream), "state init");
-  RX_CUDA(cudaMemsetAsync(rx->err, 0, sizeof(int), rx->stream), "state init");
-  RX_CUDA(cudaMemsetAsync(rx->trace_fo, 0, (size_t)rx->trace_cap * 2 * sizeof(double), rx->stream), "state init");
-  if (rx->inner)
-    RX_CUDA(cudaMemsetAsync(rx->inner, 0xff, (size_t)2 * rx->inner_cap, rx->stream), "state init");
-  // pageable source: the copy completes before cudaMemcpyAsync returns
+  const int64_t n_fo = 2 * rx->trace_cap, n_in = rx->inner ? 2 * rx->inner_cap : 0;
+  const int64_t work = std::max<int64_t>(std::max(n_fo, n_in), 2 * kEqBarrierWords);
+  const unsigned grid = (unsigned)std::min<int64_t>((work + 255) / 256, 4 * rx->sms);
+  stream_init_kernel<<<grid, 256, 0, rx->stream>>>(rx->st, (rx->T - 1) / 2, rx->m_carry, rx->err, rx->trace_fo, n_fo,
+                                                   rx->inner, n_in, rx->barrier);
+  rx->bar_set = false;
+  RX_CUDA(cudaGetLastError(), "state init");
   return RX_OK;
 }
 
@@ -545,7 +561,7 @@ rx_status rx_reserve(rx_stream *rx, int64_t max_call) {
   RX_ALLOC(rx->trace, (size_t)rx->trace_cap * 4 * kMaxTaps * 2);
   RX_ALLOC(rx->trace_fo, (size_t)rx->trace_cap * 2);
   if (rx->inner_cap > 0) RX_ALLOC(rx->inner, (size_t)2 * rx->inner_cap);
-  RX_ALLOC(rx->barrier, kEqBarrierWords);
+  RX_ALLOC(rx->barrier, 2 * kEqBarrierWords);
   RX_ALLOC(rx->err, 1);
   RX_ALLOC(rx->chunk_r, (size_t)2 * rx->chunk_cap);
   RX_ALLOC(rx->chunk_s2, (size_t)2 * rx->chunk_cap);
@@ -709,26 +725,33 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
   if (F_cdc_new - u_keep > rx->u_cap) return fail(rx, RX_EINVAL, "CDC buffer overflow (call too large for the reservation)");
   const int64_t y_keep = std::max<int64_t>(0, rx->F_out - rx->Nb - 1);
   if (new_eq - y_keep > rx->y_cap) return fail(rx, RX_EINVAL, "equaliser buffer overflow");
+  SlideArgs sl;
+  memset(&sl, 0, sizeof(sl));
+  sl.fmt = rx->fmt;
+  sl.u_stride = rx->u_cap;
+  sl.y_stride = rx->y_cap;
   if (u_keep != rx->u_base) {
-    const int64_t keep = F_cdc_old - u_keep;
-    StageTimer tm(rx, RX_STAGE_MOVE, st);
-    rx->stage_launches[RX_STAGE_MOVE] += keep > 0;
     const int nxt = 1 - rx->cur_u;
-    RX_CUDA(launch_copy_cols_fmt(u_at(rx, nxt, 0, 0), rx->u_cap, u_at(rx, rx->cur_u, 0, u_keep - rx->u_base), rx->u_cap,
-                                 keep, rx->fmt, st),
-            "slide u");
+    sl.nu = F_cdc_old - u_keep;
+    sl.u_dst = u_at(rx, nxt, 0, 0);
+    sl.u_src = u_at(rx, rx->cur_u, 0, u_keep - rx->u_base);
     rx->cur_u = nxt;
     rx->u_base = u_keep;
   }
   if (y_keep != rx->y_base) {
-    const int64_t keep = std::max<int64_t>(0, rx->F_eq - y_keep);
-    StageTimer tm(rx, RX_STAGE_MOVE, st);
-    rx->stage_launches[RX_STAGE_MOVE] += 2 * (keep > 0);
     const int nxt = 1 - rx->cur_y;
-    RX_CUDA(launch_copy_cols(rx->y[nxt], rx->y_cap, rx->y[rx->cur_y] + (y_keep - rx->y_base), rx->y_cap, keep, st), "slide y");
-    RX_CUDA(launch_copy_cols_i8(rx->bh[nxt], rx->y_cap, rx->bh[rx->cur_y] + (y_keep - rx->y_base), rx->y_cap, keep, st), "slide bhat");
+    sl.ny = std::max<int64_t>(0, rx->F_eq - y_keep);
+    sl.y_dst = rx->y[nxt];
+    sl.y_src = rx->y[rx->cur_y] + (y_keep - rx->y_base);
+    sl.b_dst = rx->bh[nxt];
+    sl.b_src = rx->bh[rx->cur_y] + (y_keep - rx->y_base);
     rx->cur_y = nxt;
     rx->y_base = y_keep;
+  }
+  if (sl.nu + sl.ny > 0) {
+    StageTimer tm(rx, RX_STAGE_MOVE, st);
+    rx->stage_launches[RX_STAGE_MOVE] += 1;
+    RX_CUDA(launch_slide(sl, st), "slide");
   }
 
   // ---------------------------------------------------------------- pieces on three streams
@@ -783,7 +806,10 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       L.trace = rx->trace;
       L.trace_fo = rx->trace_fo;
       L.trace_cap = rx->trace_cap;
-      L.barrier = rx->barrier;
+      // two counter sets in turn: each launch zeroes the other one for the next
+      L.barrier = rx->barrier + (rx->bar_set ? kEqBarrierWords : 0);
+      L.barrier_next = rx->barrier + (rx->bar_set ? 0 : kEqBarrierWords);
+      rx->bar_set = !rx->bar_set;
       L.err = rx->err;
       L.K = K;
       L.run_acq = j == 0 && run_acq;
@@ -814,7 +840,6 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       L.nblocks = eq_grid(rx);
       L.alt = L.nblocks > rx->eq_blocks;
       L.u_fmt = rx->fmt;
-      RX_CUDA(cudaMemsetAsync(rx->barrier, 0, kEqBarrierWords * sizeof(unsigned), rx->sub[1]), "barrier reset");
       StageTimer tm(rx, RX_STAGE_EQ, rx->sub[1]);
       rx->stage_launches[RX_STAGE_EQ] += 1;
       RX_CUDA(launch_eq(L, rx->sub[1]), "equaliser");

@@ -72,8 +72,9 @@ struct EqLaunch {
   float *trace;             // [trace_cap][2*2*kMaxTaps*2] wave start taps
   double *trace_fo;         // [trace_cap][2] (dw, Phi)
   int64_t trace_cap;
-  unsigned *barrier;        // [kEqCounters][kCtrStride] counters, one per 128-byte line (zeroed
-                            // before launch): [0] grid barrier after the acquisition, [1]
+  unsigned *barrier_next;   // the counters of the stream's next launch, zeroed by this one (or null)
+  unsigned *barrier;        // [kEqCounters][kCtrStride] counters, one per 128-byte line (zero
+                            // at launch): [0] grid barrier after the acquisition, [1]
                             // acquisition row pair, [2 + s] CTA arrivals of the waves in slot s
                             // (FO partials written), [2 + kWaveSlots + p] row-p arrivals (a
                             // wave's end taps written)
@@ -112,7 +113,7 @@ struct BpsLaunch {
   float *chunk_s2;          // [2][n_chunks] sum of |z - dec z|^2
   int64_t *chunk_m;         // [2][n_chunks] exclusive prefix (filled by the scan)
   int64_t *m_carry;         // [2] unwrap count carried from earlier calls
-  double *region_s2;        // [2][n_regions] sigma^2 of regions in this call
+  double *region_s2;        // [2][n_regions] 1 / sigma^2 of regions in this call
   int64_t k_lo, k_hi;       // symbols to emit [k_lo, k_hi)
   int64_t K_end;            // symbols known to exist (stream end if flushed)
   int64_t A, span;          // region layout
@@ -164,12 +165,22 @@ cudaError_t ber_run(const uint32_t *rx_bits, int64_t rx_stride, const uint32_t *
                     int32_t *sync);
 cudaError_t launch_copy_cols(float2 *dst, int64_t dst_stride, const float2 *src,
                              int64_t src_stride, int64_t n, cudaStream_t s);
-// Column copies in a storage format (fmt) and conversion to complex float.
-cudaError_t launch_copy_cols_fmt(void *dst, int64_t dst_stride, const void *src, int64_t src_stride, int64_t n,
-                                 int fmt, cudaStream_t s);
+// A stream's carried columns to the other buffer of each pair: nu samples of u (storage
+// format fmt), ny symbols of y and of the angles; strides per row, the same on both sides.
+struct SlideArgs {
+  void *u_dst;
+  const void *u_src;
+  int64_t u_stride, nu;
+  int fmt;
+  float2 *y_dst;
+  const float2 *y_src;
+  int8_t *b_dst;
+  const int8_t *b_src;
+  int64_t y_stride, ny;
+};
+cudaError_t launch_slide(const SlideArgs &a, cudaStream_t s);
+// Conversion of columns in a storage format (fmt) to complex float.
 cudaError_t launch_cols_to_f32(float2 *dst, int64_t dst_stride, const void *src, int64_t src_stride, int64_t n,
                                int fmt, cudaStream_t s);
-cudaError_t launch_copy_cols_i8(int8_t *dst, int64_t dst_stride, const int8_t *src,
-                                int64_t src_stride, int64_t n, cudaStream_t s);
 
 }  // namespace rx
