@@ -4,8 +4,8 @@
 // (Re u_i, Im u_i) -- the real form of h[i] u + g[i] conj(u), with
 // m00 = Re(h+g), m10 = Im(h+g), m11 = Re(h-g), m01 = -Im(h-g) -- so that the
 // output costs 16 FMAs and the LMS step M_i += 2 mu (Re e, Im e)^T (Re u, Im u)
-// another 16.  A segment's symbols run in order, everything in registers, on two
-// lanes (wl2_kernel: the two components of the output).  The strictly linear
+// another 16.  A segment's symbols run in order, everything in registers, on four
+// lanes (wl4_kernel; two components x two halves of the taps).  The strictly linear
 // variant keeps h complex (g = 0), which couples the components: one lane per segment
 // (wl_kernel).  Each warp stages its segments' inputs through shared memory in coalesced
 // chunks, one chunk ahead of the recursion.  Acquisition is the same code on one
@@ -146,7 +146,7 @@ template <int MB, bool HAS_Z>
 __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x4, int64_t K, int64_t s_begin,
                                                     int S, int nseg, int Wp, const WlTaps *__restrict__ taps_in,
                                                     WlTaps *__restrict__ taps_out, uint32_t *__restrict__ bits,
-                                                    float2 *__restrict__ z, float mu, const float4 *__restrict__ tail) {
+                                                    float2 *__restrict__ z, float mu, const float4 *__restrict__ tail, float4 *__restrict__ tail_next) {
   __shared__ __align__(16) float4 ring[2][WBLOCK][WROW];
   constexpr int WPS = WSUB * MB / 32;    // bit words per sub-chunk: 1 (QPSK) or 2 (16QAM)
   const int lane = threadIdx.x;
@@ -247,6 +247,7 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
     __syncwarp();   // the slot is refilled by the copy issued in the next iteration
   }
   if (live && j == nseg - 1) {
+    if (tail_next != nullptr) *tail_next = x4[K - 1];   // continues the next buffer's first regressor
     st.flush();
 #pragma unroll
     for (int i = 0; i < WT; ++i) {
@@ -260,152 +261,147 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
   }
 }
 
-// Widely-linear form on two lanes per segment (16 segments per warp).  With M_i as above,
+// Widely-linear form on four lanes per segment (8 segments per warp).  With M_i as above,
 // Re z and Im z are two recursions that share only their input: Re e updates the upper
-// rows (m00, m01) and Im e the lower ones, so lane `comp` of a pair runs component comp
-// with no exchange; every sum is formed in the order of a plain one-lane form.  A symbol is
-// one latency chain (correction, decision, error); the next symbol's dot product and the
-// tap update stand beside it, and a block's samples are read ahead.  One lane per segment
-// took 68 ns per symbol (561 us for the acquisition's 8192), four lanes with the taps
-// split as well 46 (their exchange waits on the chain), packed FP32 pairs 58, this form 41.
+// rows (m00, m01) and Im e the lower ones.  Lane 2 comp + half runs component comp over
+// the taps i = half, half + 2: its half of the dot product M u and of the look-ahead's
+// u(k-1) . u(k), one exchange each with the other half, the decision, and the update of its
+// own four entries.  Every sum is formed in the order of a plain one-lane form.  What counts
+// is a warp's instructions per symbol and what waits: the next symbol's half sums and their
+// exchange stand in front of this symbol's decision, which takes as long.  Per symbol: one
+// lane 68 ns (561 us for the acquisition's 8192), four lanes with the exchange behind the
+// decision 46, two lanes (no exchange, twice the sums) 43, this form 37.
 // The segments of a warp run in lockstep over [s0 - W, s0 + S); where one starts later or
 // ends earlier its state holds.
-struct f2x { float x, y; };              // values of the taps i, i + 1
-__device__ __forceinline__ f2x f2_pack(float lo, float hi) { return f2x{lo, hi}; }
-__device__ __forceinline__ float f2_sum(f2x v) { return v.x + v.y; }
-__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) { return f2x{a.x * b.x, a.y * b.y}; }
-__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) { return f2x{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
-
-// e' = mu_s (dec(z) - z) of one component and its Gray bits (wl_decide's).  Both levels'
-// errors are formed while |z| is compared: one select at the end of the chain.
+// e' = mu_s (dec(z) - z) of one component, with wl_decide's level: its sign and size (16QAM)
+// as flags.  Both levels' errors are formed while |z| is compared: one select at the end
+// of the chain.
 template <int MB>
-__device__ __forceinline__ float wl_error(float z, float mu_s, unsigned &b) {
+__device__ __forceinline__ float wl_error(float z, float mu_s, bool &neg, bool &outer) {
   const float mz = -mu_s * z;
+  neg = z < 0.f;
   if (MB == 2) {
-    const float d = wl_decide<2>(z, b);
-    return fmaf(mu_s, d, mz);
+    outer = false;
+    return fmaf(mu_s, neg ? -0.70710678118654752f : 0.70710678118654752f, mz);
   }
-  const bool outer = fabsf(z) > 0.63245553203367587f;      // |x sqrt 10| > 2
-  b = (z < 0.f ? 1u : 0u) | (outer ? 2u : 0u);
-  const bool pos = z >= 0.f;
-  const float e3 = fmaf(mu_s, pos ? 0.94868329805051381f : -0.94868329805051381f, mz);
-  const float e1 = fmaf(mu_s, pos ? 0.31622776601683793f : -0.31622776601683793f, mz);
+  outer = fabsf(z) > 0.63245553203367587f;                 // |x sqrt 10| > 2
+  const float e3 = fmaf(mu_s, neg ? -0.94868329805051381f : 0.94868329805051381f, mz);
+  const float e1 = fmaf(mu_s, neg ? -0.31622776601683793f : 0.31622776601683793f, mz);
   return outer ? e3 : e1;
 }
 
 template <int MB>
-struct WlRec2 {
-  f2x a01, a23, b01, b23;    // this component's row: factors of Re u (a) and Im u (b)
-  f2x r01, i01, r23, i23;    // Re, Im of the previous symbol's (u0, u1) and (u2, u3)
+struct WlRec4 {
+  float a0, a1, b0, b1;      // this component's factors of Re, Im u: taps half (a) and half + 2 (b)
+  float2 ua, ub;             // u_half, u_{half+2} of the previous symbol
   float e;                   // e' of the previous symbol (0 before the first)
 
-  // r = M(k-1) u(k) and c = u(k-1) . u(k); p = (x[2k], x[2k+1]) = (u1, u0)
-  __device__ __forceinline__ float dot(f2x vr, f2x vi) const {
-    f2x r = f2_mul(a01, vr);
-    r = f2_fma(a23, r01, r);
-    r = f2_fma(b01, vi, r);
-    r = f2_fma(b23, i01, r);
-    return f2_sum(r);
+  // this half of M(k-1) u(k); v = u_half(k), u_{half+2}(k) = u_half(k-1)
+  __device__ __forceinline__ float dot(float2 v, float2 vb) const {
+    float r = a0 * v.x;
+    r = fmaf(b0, vb.x, r);
+    r = fmaf(a1, v.y, r);
+    return fmaf(b1, vb.y, r);
   }
-  __device__ __forceinline__ float corr(f2x vr, f2x vi) const {
-    f2x c = f2_mul(r01, vr);
-    c = f2_fma(i01, vi, c);
-    c = f2_fma(r23, r01, c);
-    c = f2_fma(i23, i01, c);
-    return f2_sum(c);
+  // this half of u(k-1) . u(k)
+  static __device__ __forceinline__ float corr(float2 v, float2 p, float2 pb) {
+    float c = p.x * v.x;
+    c = fmaf(p.y, v.y, c);
+    c = fmaf(pb.x, p.x, c);
+    return fmaf(pb.y, p.y, c);
   }
-  __device__ __forceinline__ void shift(f2x vr, f2x vi) {
-    r23 = r01;
-    i23 = i01;
-    r01 = vr;
-    i01 = vi;
+  static __device__ __forceinline__ float both(float h) { return h + __shfl_xor_sync(0xffffffffu, h, 1); }
+
+  __device__ __forceinline__ void update() {
+    a0 = fmaf(e, ua.x, a0);
+    a1 = fmaf(e, ua.y, a1);
+    b0 = fmaf(e, ub.x, b0);
+    b1 = fmaf(e, ub.y, b1);
   }
 
-  __device__ __forceinline__ float step(float4 p, float mu_s, unsigned &bit) {
-    const f2x vr = f2_pack(p.z, p.x), vi = f2_pack(p.w, p.y);
-    const float z = fmaf(e, corr(vr, vi), dot(vr, vi));
+  __device__ __forceinline__ float step(float2 v, float mu_s, bool &neg, bool &outer) {
+    const float z = fmaf(e, both(corr(v, ua, ub)), both(dot(v, ua)));
     update();
-    shift(vr, vi);
-    e = wl_error<MB>(z, mu_s, bit);
+    ub = ua;
+    ua = v;
+    e = wl_error<MB>(z, mu_s, neg, outer);
     return z;
   }
 
-  // N symbols in order: the next symbol's sums in front of this one's decision.
+  // N symbols in order (v at a stride of two): each symbol's sums in front of the last one's
+  // decision.
   template <int N, class F>
-  __device__ __forceinline__ void steps(const float4 *p, float mu_s, F emit) {
-    float4 x[N];
+  __device__ __forceinline__ void steps(const float2 *p, float mu_s, F emit) {
+    float2 v[N];
+    float c[N];
 #pragma unroll
-    for (int q = 0; q < N; ++q) x[q] = p[q];
-    f2x vr = f2_pack(x[0].z, x[0].x), vi = f2_pack(x[0].w, x[0].y);
-    float r = dot(vr, vi), c = corr(vr, vi);
+    for (int q = 0; q < N; ++q) v[q] = p[2 * q];
+#pragma unroll
+    for (int q = 0; q < N; ++q) c[q] = both(corr(v[q], q > 0 ? v[q - 1] : ua, q > 1 ? v[q - 2] : (q == 1 ? ua : ub)));
+    float h = dot(v[0], ua);
+    float x = __shfl_xor_sync(0xffffffffu, h, 1);
 #pragma unroll
     for (int q = 0; q < N; ++q) {
-      const float z = fmaf(e, c, r);
+      const float z = fmaf(e, c[q], h + x);
       update();
-      shift(vr, vi);
+      ub = ua;
+      ua = v[q];
       if (q + 1 < N) {
-        vr = f2_pack(x[q + 1].z, x[q + 1].x);
-        vi = f2_pack(x[q + 1].w, x[q + 1].y);
-        r = dot(vr, vi);
-        c = corr(vr, vi);
+        h = dot(v[q + 1], ua);
+        x = __shfl_xor_sync(0xffffffffu, h, 1);
       }
-      unsigned b;
-      e = wl_error<MB>(z, mu_s, b);
-      emit(q, z, b);
+      bool neg, outer;
+      e = wl_error<MB>(z, mu_s, neg, outer);
+      emit(q, z, neg, outer);
     }
-  }
-
-  __device__ __forceinline__ void update() {
-    const f2x ee = f2_pack(e, e);
-    a01 = f2_fma(ee, r01, a01);
-    a23 = f2_fma(ee, r23, a23);
-    b01 = f2_fma(ee, i01, b01);
-    b23 = f2_fma(ee, i23, b23);
   }
 };
 
-constexpr int WSEG2 = WBLOCK / 2;        // segments per warp
+constexpr int WSEG4 = WBLOCK / 4;        // segments per warp
+// Unused dynamic shared memory of a one-segment launch (the acquisition): its warp is one
+// instruction-bound chain, and the front end's CTAs of the next buffers on the same SM take its
+// issue slots (four buffers through the whole chain: 730 us beside them, 670 alone).
+constexpr int kAcqPadSmem = 180 * 1024;
 
 template <int MB, bool HAS_Z>
-__global__ void __launch_bounds__(WBLOCK) wl2_kernel(const float4 *__restrict__ x4, int64_t K, int64_t s_begin,
+__global__ void __launch_bounds__(WBLOCK) wl4_kernel(const float4 *__restrict__ x4, int64_t K, int64_t s_begin,
                                                      int S, int nseg, int Wp, const WlTaps *__restrict__ taps_in,
                                                      WlTaps *__restrict__ taps_out, uint32_t *__restrict__ bits,
-                                                     float2 *__restrict__ z, float mu, const float4 *__restrict__ tail) {
-  __shared__ __align__(16) float4 ring[2][WSEG2][WROW];
+                                                     float2 *__restrict__ z, float mu, const float4 *__restrict__ tail, float4 *__restrict__ tail_next) {
+  __shared__ __align__(16) float4 ring[2][WSEG4][WROW];
   constexpr int WPS = WSUB * MB / 32;    // bit words per sub-chunk: 1 (QPSK) or 2 (16QAM)
   const int lane = threadIdx.x;
-  const int seg = lane >> 1, comp = lane & 1;
-  const int j = blockIdx.x * WSEG2 + seg;
+  const int seg = lane >> 2, comp = (lane >> 1) & 1, half = lane & 1;
+  const int j = blockIdx.x * WSEG4 + seg;
   const bool live = j < nseg;
   const int64_t s0 = s_begin + (int64_t)j * S;
   const int64_t s1 = s0 + S < K ? s0 + S : K;
   const int64_t base = s0 - Wp;          // symbol of the lockstep's first step
   const int64_t p0 = base > 0 ? base : 0;
-  const int64_t b_first = s_begin + (int64_t)blockIdx.x * WSEG2 * S - Wp;   // base of the warp's segment 0
+  const int64_t b_first = s_begin + (int64_t)blockIdx.x * WSEG4 * S - Wp;   // base of the warp's segment 0
   const int64_t span = (int64_t)Wp + S;
   const int64_t nch = (span + WCH - 1) / WCH;
   // chunk c of every segment: pairs base + c WCH + lane; zero outside the buffer or past the last segment
   auto issue = [&](int64_t c) {
 #pragma unroll
-    for (int q = 0; q < WSEG2; ++q) {
+    for (int q = 0; q < WSEG4; ++q) {
       const int64_t idx = b_first + (int64_t)q * S + c * WCH + lane;
-      const bool ok = blockIdx.x * WSEG2 + q < nseg && idx >= 0 && idx < K;
+      const bool ok = blockIdx.x * WSEG4 + q < nseg && idx >= 0 && idx < K;
       wl_cp16(&ring[c & 1][q][lane], ok ? (const void *)(x4 + idx) : (const void *)x4, ok ? 16 : 0);
     }
     wl_cp_commit();
   };
   issue(0);
-  WlRec2<MB> st;
-  st.a01 = f2_pack(taps_in->m[0][2 * comp], taps_in->m[1][2 * comp]);
-  st.a23 = f2_pack(taps_in->m[2][2 * comp], taps_in->m[3][2 * comp]);
-  st.b01 = f2_pack(taps_in->m[0][2 * comp + 1], taps_in->m[1][2 * comp + 1]);
-  st.b23 = f2_pack(taps_in->m[2][2 * comp + 1], taps_in->m[3][2 * comp + 1]);
-  st.r01 = st.i01 = st.r23 = st.i23 = f2_pack(0.f, 0.f);
+  WlRec4<MB> st;
+  st.a0 = taps_in->m[half][2 * comp];
+  st.a1 = taps_in->m[half][2 * comp + 1];
+  st.b0 = taps_in->m[half + 2][2 * comp];
+  st.b1 = taps_in->m[half + 2][2 * comp + 1];
+  st.ua = st.ub = make_float2(0.f, 0.f);
   st.e = 0.f;
-  if (live) {   // x[2 p0 - 1], x[2 p0 - 2]: before the buffer, the previous one's last two samples
+  if (live) {   // x[2 p0 - 1] (half 0), x[2 p0 - 2] (half 1): before the buffer, the previous one's last two samples
     const float4 h = p0 > 0 ? __ldg(&x4[p0 - 1]) : *tail;
-    st.r01 = f2_pack(h.z, h.x);
-    st.i01 = f2_pack(h.w, h.y);
+    st.ua = half ? make_float2(h.x, h.y) : make_float2(h.z, h.w);
   }
   const float mu_s = 2.f * mu;
   for (int64_t c = 0; c < nch; ++c) {
@@ -416,12 +412,12 @@ __global__ void __launch_bounds__(WBLOCK) wl2_kernel(const float4 *__restrict__ 
       wl_cp_wait<0>();
     }
     __syncwarp();
-    const float4 *row = &ring[c & 1][seg][0];
+    const float2 *row = reinterpret_cast<const float2 *>(&ring[c & 1][seg][0]) + (1 - half);
 #pragma unroll 1
     for (int h = 0; h < WCH / WSUB; ++h) {
       const int64_t t0 = c * WCH + h * WSUB;               // the same for every segment
       const int64_t start = base + t0;
-      const float4 *r = row + h * WSUB;
+      const float2 *r = row + 2 * h * WSUB;
       const bool out = t0 >= Wp;                           // Wp is a multiple of 16
       const bool whole = !live || (start >= p0 && start + WSUB <= s1);
       unsigned w[WPS];
@@ -430,21 +426,23 @@ __global__ void __launch_bounds__(WBLOCK) wl2_kernel(const float4 *__restrict__ 
       float *zo = HAS_Z ? reinterpret_cast<float *>(z + start) + comp : nullptr;
       if (t0 >= span || !__any_sync(0xffffffffu, live && start < s1)) break;
       if (__all_sync(0xffffffffu, whole)) {
-        st.template steps<WSUB>(r, mu_s, [&](int q, float zv, unsigned b) {
-          w[(q * MB) >> 5] |= b << ((q * MB) & 31);
-          if (HAS_Z && out && live) zo[2 * q] = zv;
+        st.template steps<WSUB>(r, mu_s, [&](int q, float zv, bool neg, bool outer) {
+          if (neg) w[(q * MB) >> 5] |= 1u << ((q * MB) & 31);
+          if (MB == 4 && outer) w[(q * MB) >> 5] |= 2u << ((q * MB) & 31);
+          if (HAS_Z && out && live && half == 0) zo[2 * q] = zv;
         });
       } else {
 #pragma unroll 1
         for (int q = 0; q < WSUB; ++q) {
-          unsigned b;
-          WlRec2<MB> nx = st;
-          const float zv = nx.step(r[q], mu_s, b);
+          bool neg, outer;
+          WlRec4<MB> nx = st;
+          const float zv = nx.step(r[2 * q], mu_s, neg, outer);
+          const unsigned b = (neg ? 1u : 0u) | (outer ? 2u : 0u);
           if (live && start + q >= p0 && start + q < s1) {
             st = nx;
             if (MB == 2 || q < 8) w[0] |= b << ((q * MB) & 31);
             else w[WPS - 1] |= b << ((q * MB) & 31);
-            if (HAS_Z && out) zo[2 * q] = zv;
+            if (HAS_Z && out && half == 0) zo[2 * q] = zv;
           }
         }
       }
@@ -452,38 +450,42 @@ __global__ void __launch_bounds__(WBLOCK) wl2_kernel(const float4 *__restrict__ 
 #pragma unroll
         for (int t = 0; t < WPS; ++t) {
           w[t] <<= comp * (MB / 2);
-          w[t] |= __shfl_xor_sync(0xffffffffu, w[t], 1);
+          w[t] |= __shfl_xor_sync(0xffffffffu, w[t], 2);
         }
         const int64_t nv = s1 - start;
         const int nw = (int)((min(nv, (int64_t)WSUB) * MB + 31) >> 5);
-        if (live && nv > 0 && comp < WPS && comp < nw) bits[((start * MB) >> 5) + comp] = comp == 0 ? w[0] : w[WPS - 1];
+        const int wi = lane & 3;
+        if (live && nv > 0 && wi < WPS && wi < nw) bits[((start * MB) >> 5) + wi] = wi == 0 ? w[0] : w[WPS - 1];
       }
     }
     __syncwarp();   // the slot is refilled by the copy issued in the next iteration
   }
   wl_cp_wait<0>();
   if (live && j == nseg - 1) {
+    if (tail_next != nullptr && (lane & 3) == 0) *tail_next = x4[K - 1];   // continues the next buffer's first regressor
     st.update();    // the one still pending after the last symbol
-    const f2x row[4] = {st.a01, st.a23, st.b01, st.b23};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float lo = row[q].x, hi = row[q].y;
-      taps_out->m[2 * (q & 1)][2 * comp + (q >> 1)] = lo;
-      taps_out->m[2 * (q & 1) + 1][2 * comp + (q >> 1)] = hi;
-    }
+    taps_out->m[half][2 * comp] = st.a0;
+    taps_out->m[half][2 * comp + 1] = st.a1;
+    taps_out->m[half + 2][2 * comp] = st.b0;
+    taps_out->m[half + 2][2 * comp + 1] = st.b1;
   }
 }
 
 // one launch, modulation, form and the optional output as template arguments
 template <int MB, bool LINEAR, bool HAS_Z>
 void launch_wl_k(cudaStream_t s, const float4 *x4, int64_t K, int64_t s_begin, int S, int nseg, int Wp, const WlTaps *tin,
-                 WlTaps *tout, uint32_t *bits, float2 *z, float mu, const float4 *tail) {
+                 WlTaps *tout, uint32_t *bits, float2 *z, float mu, const float4 *tail, float4 *tail_next) {
+  int pad = 0;
+  if (!LINEAR && nseg == 1 && kAcqPadSmem > 0) {
+    pad = kAcqPadSmem;
+    cudaFuncSetAttribute(wl4_kernel<MB, HAS_Z>, cudaFuncAttributeMaxDynamicSharedMemorySize, pad);
+  }
   if constexpr (LINEAR)
     wl_kernel<MB, HAS_Z><<<(unsigned)((nseg + WBLOCK - 1) / WBLOCK), WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout,
-                                                                                     bits, z, mu, tail);
+                                                                                     bits, z, mu, tail, tail_next);
   else
-    wl2_kernel<MB, HAS_Z><<<(unsigned)((nseg + WSEG2 - 1) / WSEG2), WBLOCK, 0, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout,
-                                                                                    bits, z, mu, tail);
+    wl4_kernel<MB, HAS_Z><<<(unsigned)((nseg + WSEG4 - 1) / WSEG4), WBLOCK, pad, s>>>(x4, K, s_begin, S, nseg, Wp, tin, tout,
+                                                                                    bits, z, mu, tail, tail_next);
 }
 
 template <int MB, bool LINEAR, class... Args>
@@ -501,6 +503,12 @@ cudaError_t launch_wl(int mb, bool linear, bool has_z, Args... args) {
   return cudaGetLastError();
 }
 
+// Start state on the stream, by value: nothing to wait for.
+__global__ void wl_start_kernel(WlTaps *dev, WlTaps start, float4 *tail) {
+  dev[0] = start;
+  tail[0] = make_float4(0.f, 0.f, 0.f, 0.f);
+}
+
 }  // namespace
 }  // namespace rx
 
@@ -516,7 +524,8 @@ struct rx_wl {
   bool acquired = false;
   WlTaps start{};            // host copy of the start taps (matrix form)
   WlTaps *dev = nullptr;     // [0], [1]: wave-start taps ping-pong; [2]: acquisition end
-  float4 *tail = nullptr;    // the previous buffer's last two samples (zero for the first)
+  float4 *tail = nullptr;    // [2] the previous buffer's last two samples (zero for the first), by `cur`
+  bool start_pending = false;   // a reset's start state may still be on its way
   int cur = 0;               // which of dev[0..1] holds the taps for the next call
   cudaStream_t stream = nullptr;
   bool profile = false;
@@ -555,11 +564,12 @@ void from_matrix(const WlTaps &o, double *t) {
   }
 }
 
-rx_status upload_start(rx_wl *w) {
-  cudaError_t e = cudaMemcpyAsync(&w->dev[0], &w->start, sizeof(WlTaps), cudaMemcpyHostToDevice, w->stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(w->tail, 0, sizeof(float4), w->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);
-  if (e != cudaSuccess) return wfail(w, RX_ECUDA, std::string("taps upload: ") + cudaGetErrorString(e));
+rx_status upload_start(rx_wl *w, bool wait) {
+  wl_start_kernel<<<1, 1, 0, w->stream>>>(w->dev, w->start, w->tail);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && wait) e = cudaStreamSynchronize(w->stream);
+  if (e != cudaSuccess) return wfail(w, RX_ECUDA, std::string("start taps: ") + cudaGetErrorString(e));
+  w->start_pending = !wait;
   w->cur = 0;
   return RX_OK;
 }
@@ -589,13 +599,13 @@ rx_status rx_wl_create(rx_wl **out, int mod_bits, int ntaps, int64_t max_symbols
   double t[4 * WT] = {0};
   t[2 * WC] = 1.0;
   w->start = to_matrix(t);
-  if (cudaMalloc(&w->dev, 3 * sizeof(WlTaps)) != cudaSuccess || cudaMalloc(&w->tail, sizeof(float4)) != cudaSuccess) {
+  if (cudaMalloc(&w->dev, 3 * sizeof(WlTaps)) != cudaSuccess || cudaMalloc(&w->tail, 2 * sizeof(float4)) != cudaSuccess) {
     cudaGetLastError();
     cudaFree(w->dev);
     delete w;
     return RX_ENOMEM;
   }
-  if (upload_start(w) != RX_OK) {
+  if (upload_start(w, true) != RX_OK) {
     cudaFree(w->dev);
     cudaFree(w->tail);
     delete w;
@@ -649,6 +659,12 @@ rx_status rx_wl_get_param(rx_wl *w, int key, double *v) {
 
 rx_status rx_wl_set_cuda_stream(rx_wl *w, void *s) {
   if (!w) return RX_EINVAL;
+  // a reset's start state on the old stream comes before work on the new one
+  if (w->start_pending && (cudaStream_t)s != w->stream) {
+    const cudaError_t e = cudaStreamSynchronize(w->stream);
+    if (e != cudaSuccess) return wfail(w, RX_ECUDA, std::string("stream change: ") + cudaGetErrorString(e));
+    w->start_pending = false;
+  }
   w->stream = (cudaStream_t)s;
   return RX_OK;
 }
@@ -662,7 +678,7 @@ rx_status rx_wl_set_taps(rx_wl *w, const float *taps) {
     t[i] = taps[i];
   }
   w->start = to_matrix(t);
-  return upload_start(w);
+  return upload_start(w, true);
 }
 
 rx_status rx_wl_get_taps(rx_wl *w, double *taps) {
@@ -697,7 +713,7 @@ rx_status rx_wl_process(rx_wl *w, const float *x, int64_t n, uint32_t *bits, flo
     a0 = std::min<int64_t>(w->A, K);
     if (a0 > 0) {
       e = launch_wl(w->mb, w->linear, z2 != nullptr, w->stream, x4, K, (int64_t)0, (int)a0, 1, 0, from, &w->dev[2], bits, z2,
-                    (float)w->mu, (const float4 *)w->tail);
+                    (float)w->mu, (const float4 *)w->tail + w->cur, a0 == K ? w->tail + 1 - w->cur : nullptr);
       from = &w->dev[2];
     }
     w->acquired = true;
@@ -708,15 +724,13 @@ rx_status rx_wl_process(rx_wl *w, const float *x, int64_t n, uint32_t *bits, flo
   if (e == cudaSuccess && rest > 0) {
     const int64_t nseg = (rest + w->S - 1) / w->S;
     e = launch_wl(w->mb, w->linear, z2 != nullptr, w->stream, x4, K, a0, w->S, (int)nseg, w->W, from, &w->dev[nxt], bits,
-                  z2, (float)w->mu, (const float4 *)w->tail);
+                  z2, (float)w->mu, (const float4 *)w->tail + w->cur, w->tail + nxt);
     w->cur = nxt;
   } else if (e == cudaSuccess && a0 > 0) {
     // the whole call was acquisition: its end taps start the next call
     e = cudaMemcpyAsync(&w->dev[nxt], &w->dev[2], sizeof(WlTaps), cudaMemcpyDeviceToDevice, w->stream);
     w->cur = nxt;
   }
-  // this buffer's last two samples continue the next buffer's first regressor
-  if (e == cudaSuccess) e = cudaMemcpyAsync(w->tail, x4 + (K - 1), sizeof(float4), cudaMemcpyDeviceToDevice, w->stream);
   if (ev[2]) {
     cudaEventRecord(ev[2], w->stream);
     w->pending.push_back({0, {ev[0], ev[1]}});
@@ -730,7 +744,7 @@ rx_status rx_wl_reset(rx_wl *w) {
   if (!w) return RX_EINVAL;
   w->started = false;
   w->acquired = false;
-  return upload_start(w);
+  return upload_start(w, false);
 }
 
 rx_status rx_wl_profile(rx_wl *w, int on, double *ms, int reset) {
