@@ -23,12 +23,12 @@ __device__ __forceinline__ float2 cmul_mi(float2 a) { return make_float2(a.y, -a
 // (x >= 0 decides the positive side; 16QAM |x sqrt10| > 2 is the outer level).
 template <int MB>
 __device__ __forceinline__ float qam_level(float x) {
-  if (MB == 2) {
-    return x >= 0.f ? 0.70710678118654752f : -0.70710678118654752f;
-  } else {
-    const float l = fabsf(x * 3.16227766016837933f) > 2.f ? 3.f * 0.31622776601683793f : 0.31622776601683793f;
-    return x >= 0.f ? l : -l;
-  }
+  // the sign bit of x + 0 (a negative zero decides positive); both 16QAM levels get it
+  // while |x| is compared, so a decision is one select behind the comparison
+  const float xs = x + 0.f;
+  if (MB == 2) return copysignf(0.70710678118654752f, xs);
+  const float l3 = copysignf(3.f * 0.31622776601683793f, xs), l1 = copysignf(0.31622776601683793f, xs);
+  return fabsf(x * 3.16227766016837933f) > 2.f ? l3 : l1;
 }
 
 template <int MB>

@@ -763,8 +763,9 @@ __device__ __forceinline__ void run_span(const Hot hot, EqSmem<NW> &sm, const Sp
         tot = make_float2(((gs[0].x + gs[1].x) + (gs[2].x + gs[3].x)) + ((gs[4 % NW].x + gs[5 % NW].x) + (gs[6 % NW].x + gs[7 % NW].x)),
                           ((gs[0].y + gs[1].y) + (gs[2].y + gs[3].y)) + ((gs[4 % NW].y + gs[5 % NW].y) + (gs[6 % NW].y + gs[7 % NW].y)));
       }
-      own.x = tap_ok ? __fmaf_rn(-mu, tot.x, own.x) : own.x;
-      own.y = tap_ok ? __fmaf_rn(-mu, tot.y, own.y) : own.y;
+      // (the sixteenth tap's samples are zero in a whole block: so is its sum)
+      own.x = FULLB || tap_ok ? __fmaf_rn(-mu, tot.x, own.x) : own.x;
+      own.y = FULLB || tap_ok ? __fmaf_rn(-mu, tot.y, own.y) : own.y;
       gather_taps<NW>(h, own, ln);
       d_on = act && ln.part == 0 && s0 >= emit && s0 + kl >= pair_lo && s0 + kl < pair_hi;
       d_yv = yv;

@@ -336,14 +336,14 @@ unsigned char *u_at(rx_stream *rx, int b, int p, int64_t n) {
 // Region layout: region 0 = [0, A), region r >= 1 = [A + (r-1) span, A + r span).
 // Pieces of a call of n waves when the caller names none.  A piece hides what comes before
 // and after it (the first piece's CDC and the last one's BPS stay in the open: about
-// 4.7 us per wave of the piece) and costs the equaliser's start and drain, about 20 us of a
+// 4 us per wave of the piece) and costs the equaliser's start and drain, 13 to 16 us of a
 // launch: the sum is least near sqrt(n) / 2 pieces, and pieces also wait on their CDC
-// beside the equaliser, which moves the measured minimum to sqrt(n) / 3 (10 GBd QPSK, 512
-// waves: 1, 3, 6, 12, 20 pieces 10.47, 9.35, 9.23, 9.43, 9.47 ms; 32 GBd 16QAM, 31 waves:
-// 1, 2, 4, 12 pieces 1082, 1033, 1040, 1190 us; 21 waves: 1, 2, 4, 12 pieces 802, 775, 796,
-// 930 us; calls of 9 waves: 1, 2, 12 pieces 1636, 1789, 2043 us).
+// beside the equaliser, so the line lies a little below (10 GBd QPSK, 512 waves: 3, 5, 6, 8,
+// 10 pieces 9.89, 9.48, 9.43, 9.38, 9.32 ms; 32 GBd 16QAM, 31 waves: 1, 2, 4, 12 pieces
+// 1082, 1033, 1040, 1190 us; 21 waves: 1, 2, 4, 12 pieces 802, 775, 796, 930 us; calls of 9
+// waves: 1, 2, 12 pieces 1636, 1789, 2043 us).
 int auto_pieces(const rx_stream *rx, int64_t n) {
-  return (int)std::min<double>(rx->pieces, std::max(1.0, floor(sqrt((double)n) / 3.0 + 0.5)));
+  return (int)std::min<double>(rx->pieces, std::max(1.0, floor(0.4 * sqrt((double)n) + 0.5)));
 }
 
 // Symbols per BPS chunk (one warp each).  A chunk's pass is one chain of 32-symbol blocks
