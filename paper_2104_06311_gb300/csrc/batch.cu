@@ -28,10 +28,9 @@
 // output sample.  Team sizes come from a cost model of the equaliser
 // schedule: a channel's time is its acquisition (A / B_u update steps, one
 // CTA pair) plus, per wave, ceil(P / pairs) passes of (S + W) / B_u steps and
-// a fixed wave overhead, times the step cost of its format (a 16QAM step costs
-// about 1.08 QPSK steps: its inner-BPS distance is longer); pairs go one at a
-// time to the channel whose time is currently largest, within the co-resident
-// CTA budget of the launch.
+// a fixed wave overhead (a 16QAM step takes as long as a QPSK one); the channel whose time is
+// currently largest takes the pairs that save it a pass, within the co-resident CTA
+// budget of the launch.
 #include <stdio.h>
 #include <stdlib.h>
 #include <string.h>
@@ -56,8 +55,6 @@ constexpr int64_t kNcma = 8192, kAcqMin = 16384, kBlockSamples = 65536;
 constexpr double kMu = 1e-3, kRolloff = 0.1, kLamNm = 1550.0, kFoSmooth = 16.0;
 constexpr int kMaxChannels = 4096;
 constexpr int kWaveOverheadSteps = 8;   // cost model: grid barrier + FO fold per wave
-constexpr double kStep16qam = 1.075;     // cost model: 16QAM update step / QPSK step (fit to per-team
-                                        // end times of a 64-channel batch)
 
 struct Chan {
   rx_chan_cfg cfg;
@@ -339,8 +336,7 @@ double eq_cost(const Chan &c, int pairs) {
   const int64_t n_seg = c.K_cap > A ? (c.K_cap - A + kS - 1) / kS : 0;
   const int64_t waves = (n_seg + c.P - 1) / c.P;
   const int64_t passes = (c.P + pairs - 1) / pairs;
-  const double step = c.cfg.mod_bits == 4 ? kStep16qam : 1.0;
-  return step * ((double)(A / kBu) + (double)waves * (double)(passes * ((kS + kW) / kBu) + kWaveOverheadSteps));
+  return ((double)(A / kBu) + (double)waves * (double)(passes * ((kS + kW) / kBu) + kWaveOverheadSteps));
 }
 
 rx_status check_device_error(rx_batch *b, bool wait) {
@@ -572,20 +568,19 @@ rx_status rx_batch_create(rx_batch **out, int n_ch, const rx_chan_cfg *cfgs) {
   }
   std::vector<int> pairs(n_ch, 1);
   int left = budget / 2 - n_ch;
-  while (left > 0) {
-    int pick = -1;
-    double worst = -1;
-    for (int i = 0; i < n_ch; ++i) {
-      if (pairs[i] >= b->ch[i].P) continue;
-      const double t = eq_cost(b->ch[i], pairs[i]);
-      if (t > worst && eq_cost(b->ch[i], pairs[i] + 1) < t) {
-        worst = t;
-        pick = i;
-      }
-    }
-    if (pick < 0) break;
-    ++pairs[pick];
-    --left;
+  while (true) {
+    // the channel that ends last takes the pairs that save it a whole pass per wave (one more
+    // often saves none: 32 segments take four passes with 8, 9 and 10 pairs); when it can have
+    // no more, more for the others would only share its SMs
+    int pick = 0;
+    for (int i = 1; i < n_ch; ++i)
+      if (eq_cost(b->ch[i], pairs[i]) > eq_cost(b->ch[pick], pairs[pick])) pick = i;
+    const int P = b->ch[pick].P, passes = (P + pairs[pick] - 1) / pairs[pick];
+    if (passes == 1) break;
+    const int need = (P + passes - 2) / (passes - 1) - pairs[pick];
+    if (need > left || eq_cost(b->ch[pick], pairs[pick] + need) >= eq_cost(b->ch[pick], pairs[pick])) break;
+    pairs[pick] += need;
+    left -= need;
   }
   std::vector<int2> team;
   for (int i = 0; i < n_ch; ++i) {
