@@ -452,7 +452,8 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_demap(BpsLaunch L) {
     unsigned v = 0;
     const int64_t jo = k - L.out_first;
     if (valid) {
-      z = cmul(yk, make_float2(rc, rs));
+      // (placed products: the symbols' rounding does not move with the compiler's contraction)
+      z = make_float2(__fmaf_rn(yk.x, rc, -__fmul_rn(yk.y, rs)), __fmaf_rn(yk.x, rs, __fmul_rn(yk.y, rc)));
       switch ((int)(((mk % 4) + 4) % 4)) {  // (-j)^m
         case 1: z = make_float2(z.y, -z.x); break;
         case 2: z = make_float2(-z.x, -z.y); break;
