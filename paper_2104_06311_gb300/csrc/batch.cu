@@ -14,7 +14,7 @@
 //            segment slot) that runs its acquisition and its segment waves
 //            and synchronises on the channel's own barrier words;
 //   BPS      pass 1 / unwrap scan / demap launches per channel;
-// the per-channel CDC and BPS launches spread over four side streams
+// the per-channel CDC and BPS launches spread over twelve side streams
 // (longest channel first onto the least loaded; fork and join by events on
 // the bound stream), so that the many short launches of small channels
 // overlap; from the second call with the same pointers and sizes the whole
@@ -174,7 +174,9 @@ struct rx_batch {
   cudaStream_t cap_stream = nullptr;         // graph capture only
   // side streams: the per-channel CDC and BPS launches, spread over them so
   // that the small channels' launches overlap (fork / join by events)
-  static constexpr int kSide = 4;
+  // (4, 8, 12, 16 streams: 64 channels 6.41, 6.19, 6.19, 6.21 ms, 24 channels 1069, 1026, 993,
+  // 987 us, 6 channels 417, 387, 387, 390 us)
+  static constexpr int kSide = 12;
   cudaStream_t side[kSide] = {};
   cudaEvent_t ev_fork = nullptr, ev_join[kSide] = {};
   bool use_graph = true;
@@ -375,15 +377,16 @@ struct BStage {
   }
 };
 
-// The side streams start after everything enqueued on s so far.
-// SMs a channel's CDC launch may fill: the side streams share the device.
+// SMs a channel's CDC launch may fill: half the device (a persistent launch on a share of
+// 1 / kSide of it ends long after the last small channel's).
 int side_sm_budget() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  return std::max(1, sms / rx_batch::kSide);
+  return std::max(1, sms / 2);
 }
 
+// The side streams start after everything enqueued on s so far.
 cudaError_t side_fork(rx_batch *b, cudaStream_t s) {
   cudaError_t e = cudaEventRecord(b->ev_fork, s);
   for (int k = 0; k < rx_batch::kSide && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(b->side[k], b->ev_fork, 0);
