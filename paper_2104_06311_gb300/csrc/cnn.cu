@@ -81,6 +81,9 @@ struct ConvArgs {
   bf16 *dout;
   double *loss;
   float inv4k;
+  // the first kernel of a training pass zeroes what later ones add to
+  float *zero;
+  int64_t n_zero;
 };
 
 template <int CIN, int COUT, int EPI>
@@ -548,6 +551,10 @@ __global__ void __launch_bounds__(TC_M) edge_in_kernel(const __grid_constant__ C
   const int64_t n_tiles = (a.K + TC_M - 1) / TC_M;
   tc_grid_wait();
   if (tid == 0) tc_grid_trigger();
+  if (a.zero) {
+    for (int64_t i = (int64_t)blockIdx.x * TC_M + tid; i < a.n_zero; i += (int64_t)gridDim.x * TC_M) a.zero[i] = 0.f;
+    if (blockIdx.x == 0 && tid == 0) *a.loss = 0.0;
+  }
   const unsigned long long y0 = tc_desc(smem_u32(op.y), smem_u32(op.zero) - smem_u32(op.y), 128u);
   const unsigned long long w0 = tc_desc(smem_u32(op.w), smem_u32(op.zero) - smem_u32(op.w), 128u);
   // feature row of symbol n as four BF16 (zero outside the sequence)
@@ -1452,9 +1459,14 @@ rx_status check_sym(rx_cnn *c, const float *p, int64_t stride, int64_t K, const 
   return RX_OK;
 }
 
-// Forward pass; with t, also the loss and dJ/dy.  y may be NULL.
-rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, const float *t, int64_t ts, int64_t K) {
+// Forward pass; with t, also the loss and dJ/dy, and G and the loss zeroed first.  y may be NULL.
+rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, const float *t, int64_t ts, int64_t K,
+                  float *G) {
   if (!c->use_tc) {
+    if (t) {
+      CX_CUDA(cudaMemsetAsync(c->loss, 0, sizeof(double), c->stream), "loss");
+      CX_CUDA(cudaMemsetAsync(G, 0, (size_t)c->n_params * sizeof(float), c->stream), "zero grads");
+    }
     const int g = (int)std::min<int64_t>((K + 255) / 256, 4 * c->sms);
     features_kernel<<<std::max(1, g), 256, 0, c->stream>>>(reinterpret_cast<const float2 *>(z), zs, K, c->x0);
     CX_CUDA(cudaGetLastError(), "features");
@@ -1473,6 +1485,11 @@ rx_status forward(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t ys, c
       a.in = l == 0 ? c->x0 : c->h[l - 1];
       a.out = c->h[l];
       if (l == 0 && c->use_tc) {
+        if (t) {
+          a.zero = G;
+          a.n_zero = c->n_params;
+          a.loss = c->loss;
+        }
         CX_CUDA((launch_edge_in<true, EPI_RELU>(c, a, c->wtc_f[l], false)), "conv (first)");
       } else if (l == 0) {
         CX_CUDA((launch_conv<FEATP, CH, EPI_RELU>(c, a)), "conv");
@@ -1660,9 +1677,7 @@ rx_status timed_out(rx_cnn *c) { return cfail(c, RX_ETIMEOUT, "a bounded device 
 
 // Forward and backward pass: the loss in c->res, the gradients in G.
 rx_status gradients(rx_cnn *c, const float *z, int64_t zs, const float *t, int64_t ts, int64_t K, float *G) {
-  CX_CUDA(cudaMemsetAsync(c->loss, 0, sizeof(double), c->stream), "loss");
-  CX_CUDA(cudaMemsetAsync(G, 0, (size_t)c->n_params * sizeof(float), c->stream), "zero grads");
-  const rx_status s = forward(c, z, zs, nullptr, 0, t, ts, K);
+  const rx_status s = forward(c, z, zs, nullptr, 0, t, ts, K, G);
   return s == RX_OK ? backward(c, z, zs, K, G) : s;
 }
 
@@ -1701,7 +1716,7 @@ rx_status rx_cnn_apply(rx_cnn *c, const float *z, int64_t zs, float *y, int64_t 
   rx_status s = check_sym(c, z, zs, K, "input");
   if (s == RX_OK) s = check_sym(c, y, ys, K, "output");
   if (s != RX_OK) return s;
-  return forward(c, z, zs, y, ys, nullptr, 0, K);
+  return forward(c, z, zs, y, ys, nullptr, 0, K, nullptr);
 }
 
 rx_status rx_cnn_grads(rx_cnn *c, const float *z, int64_t zs, const float *t, int64_t ts, int64_t K,
