@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
   __shared__ float amp[2 * KH];                // a of the kept samples, lo + 256 on
   const int t = threadIdx.x;
   if ((int)blockIdx.x >= n_pairs) {
+    asm volatile("griddepcontrol.wait;\n" ::: "memory");
     const int j = ((int)blockIdx.x - n_pairs) * KT + t;
     if (j < KHIST) hist_next[j] = kk_intensity(src, src.pos + src.n - KHIST + j);   // before the stream start: never read
     return;
@@ -143,6 +144,9 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
     }
     __syncthreads();
   }
+  // launched while the kernel in front drains: its results, and the scratch it reads, from here on
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const int w0 = 2 * blockIdx.x;
   const bool two = w0 + 1 < nwin;
   const int64_t lo = e0 + (int64_t)w0 * KH - KH / 2;          // first sample of window w0
@@ -223,6 +227,8 @@ __global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *__restr
   const int64_t i = i0 + blockIdx.x;
   const int64_t lo = i * S - V / 2;
   float2 x[16];
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const float2 *src = E + (lo - e0) + t;
 #pragma unroll
   for (int q = 0; q < 16; ++q) x[q] = src[KT * q];
@@ -397,6 +403,22 @@ namespace {
 
 int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
+// A launch whose CTAs may be placed while the kernel in front of it drains (they wait for
+// its end themselves, before they touch memory that it uses).
+template <class... KArgs, class... Args>
+cudaError_t launch_overlapped(bool overlap, void (*fn)(KArgs...), unsigned grid, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(KT);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
 // Output samples [pos - KDELAY, pos - KDELAY + no) of the stream whose input is
 // known on [start, end): Hilbert windows over the field range with KEDGE on each
 // side, then the static filter's windows over the output range.
@@ -410,19 +432,18 @@ rx_status kk_run(rx_kk *k, const KkSrc &src, int64_t no, float *y, float *field)
   const int nwin = (int)((no + 2 * KEDGE) / KH);
   const int n_pairs = (nwin + 1) / 2;
   const unsigned grid = (unsigned)(n_pairs + (src.n > 0 ? KHIST / KT : 0));   // + the history's copy
-  if (src.dtype == RX_KK_I8)
-    kk_hilbert_kernel<true><<<grid, KT, 0, k->stream>>>(src, e0, nwin, n_pairs, k->tw, k->inc_q, k->E, k->hist[1 - k->cur]);
-  else
-    kk_hilbert_kernel<false><<<grid, KT, 0, k->stream>>>(src, e0, nwin, n_pairs, k->tw, k->inc_q, k->E, k->hist[1 - k->cur]);
-  cudaError_t e = cudaGetLastError();
+  const auto hilbert = src.dtype == RX_KK_I8 ? kk_hilbert_kernel<true> : kk_hilbert_kernel<false>;
+  // (a buffer's first stage is not: its CTAs, placed early, keep the equaliser's acquisition on
+  // another stream from finding an SM, 543 -> 589 us over four buffers; the flush is small)
+  cudaError_t e = launch_overlapped(src.n == 0, hilbert, grid, k->stream, src, e0, nwin, n_pairs, (const float2 *)k->tw, k->inc_q, k->E,
+                                    k->hist[1 - k->cur]);
   if (ev[1]) cudaEventRecord(ev[1], k->stream);
   const int S = KN - k->V;
   const int64_t i0 = floor_div(o0, S), i1 = floor_div(o0 + no - 1, S);
   if (e == cudaSuccess) {
-    kk_filter_kernel<<<(unsigned)(i1 - i0 + 1), KT, 0, k->stream>>>(
-        k->E, e0, i0, o0, no, k->start, k->V, k->H, k->tw, k->tw2, reinterpret_cast<float2 *>(y),
-        reinterpret_cast<float2 *>(field));
-    e = cudaGetLastError();
+    e = launch_overlapped(true, kk_filter_kernel, (unsigned)(i1 - i0 + 1), k->stream, (const float2 *)k->E, e0, i0, o0, no, k->start,
+                          k->V, (const float2 *)k->H, (const float2 *)k->tw, (const float2 *)k->tw2,
+                          reinterpret_cast<float2 *>(y), reinterpret_cast<float2 *>(field));
   }
   if (ev[2]) {
     cudaEventRecord(ev[2], k->stream);
