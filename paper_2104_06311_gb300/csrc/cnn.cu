@@ -15,7 +15,8 @@
 // gradient dW[k][ci][co] = sum_n in[n + k - 7][ci] dz[n][co] is a GEMM with
 // the symbols as the reduction dimension: CTAs own (symbol chunk, 3 taps),
 // read both operands transposed by ldmatrix.trans, and add their partial
-// sums into the FP32 gradient with atomics.
+// sums into the FP32 gradient with atomics.  This mma.sync form runs when tcgen05 is
+// switched off (RX_CNN_OPT_TCGEN05 = 0); the default form follows below it.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
@@ -204,7 +205,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const ConvArgs a) {
 // doubles the operand reads that bound an MMA of N = 64 (4 KB of A per 32 cycles of
 // math).  15 taps x 4 groups of 16 channels = 60 MMAs per tile into one of two
 // accumulators.  The output goes through swizzled shared memory to one TMA store per
-// warp (whole 128-byte rows, clipped at the sequence end).
+// warp (whole 128-byte rows, clipped at the sequence end).  Bound by shared memory: 48
+// cycles of operand reads per MMA, 2880 per tile, and the tile's own traffic through the
+// same port; 2^20 symbols 107 us a layer (181 with unswizzled operands, descriptors built
+// per MMA and one CTA barrier per tile), 2^14 symbols 7.2 us (8.7).
 //
 // 4 -> 64 layers (edge_in_kernel: the first layer from the features, and dJ/dh of the
 // last one from dJ/dy): a feature row is 16 bytes of shared memory (4 values, 4 zeros), so
@@ -218,7 +222,8 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const ConvArgs a) {
 // P[m][4 t + c] = sum_ci h[m][ci] W[t][ci][c] (4 MMAs per tile, N = 64), and
 // out[n][c] = sum_t P[n + t - 7][4 t + c] is 15 float4 additions per symbol.  A tile of
 // 128 rows gives 114 symbols.  Both edge kernels are bound by the 128-byte rows they
-// write or read; several CTAs share an SM to overlap their phases.
+// write or read and the latency of their phases; six and four CTAs share an SM: 39 and 47 us
+// at 2^20 symbols (mma.sync 182 and 269).
 constexpr int TC_M = 128;                      // rows per tile (one MMA M)
 constexpr int TC_ROWS = TC_M + 2 * HALF;       // 142 rows per TMA box
 constexpr int TC_STAGES = 3;
@@ -783,7 +788,8 @@ __global__ void pack_tc_kernel(const float *__restrict__ W, int ci_true, int co_
 // in shared memory as pairs (x[m], x[m+1]) of 16 bytes: a core matrix (8 of M = 2 taps, 8
 // symbols) is 8 successive pairs, the next two taps are two pairs on.
 //
-// A CTA adds its part to the FP32 gradient with 16-byte atomics at the end.
+// A CTA adds its part to the FP32 gradient with 16-byte atomics at the end.  Four layers of
+// 2^14 symbols 19 us (four mma.sync launches 43).
 constexpr int DW_STAGES = 2;
 constexpr int DW_PAIRS = 2;                          // tap pairs per CTA of a hidden layer
 constexpr int DW_GROUPS = (KS + 1) / (2 * DW_PAIRS); // CTAs per chunk

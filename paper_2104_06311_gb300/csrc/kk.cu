@@ -121,7 +121,8 @@ __device__ __forceinline__ void kk_fft1024(float2 (&x)[16], int t, float2 *b0, f
 // samples on, so a thread's samples t + 64 i (i < 24) serve both.
 // CTAs from n_pairs on copy the input history for the next buffer (hist_next): the
 // intensities of stream samples [pos + n - KHIST, pos + n).
-// Bound by instructions (two 1024-point FFTs, a sine and cosine per sample).
+// Bound by the latency of its loads (samples, twiddles) at 24 warps per SM, 46 % of the issue
+// slots busy: 2^22 8-bit samples 46 us (81 with eight shared-memory crossings per pair).
 template <bool I8>
 __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e0, int nwin, int n_pairs,
                                                             const float2 *__restrict__ tw, unsigned long long inc_q,
@@ -216,6 +217,8 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
 // output samples t in [i S, i S + S) inside [o0, o0 + no) at 2 samples/symbol to
 // y[(t - o0)/2] (zero before the stream start); optionally the field itself to
 // field[t - o0] for every t of the range.
+// Bound by load and shared-memory latency: 2^22 samples 43 us (52 with 32 threads, staged loads
+// and seven crossings); 14 or 16 CTAs per SM with one buffer measured the same.
 __global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *__restrict__ E, int64_t e0, int64_t i0, int64_t o0,
                                                        int64_t no, int64_t start, int V,
                                                        const float2 *__restrict__ H, const float2 *__restrict__ tw,
