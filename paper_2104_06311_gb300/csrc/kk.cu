@@ -63,6 +63,15 @@ __device__ __forceinline__ float kk_intensity(const KkSrc &src, int64_t s) {
   return src.hist[s - (src.pos - KHIST)];
 }
 
+// A load of what the kernel in front of an overlapped launch writes: coherent, and kept behind
+// griddepcontrol.wait (a const __restrict__ pointer or __ldg would let the compiler take it for
+// read-only data of the whole kernel, whose life begins while that kernel still writes).
+__device__ __forceinline__ float2 kk_load_behind_wait(const float2 *p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+
 // ---- transforms of 64 threads: x[i] is element t + 64 i
 constexpr int KT = 64;
 constexpr int KBUF = KN + KN / 16;       // one float2 of padding per 16: unit- and 16-strided accesses conflict-free
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
 // field[t - o0] for every t of the range.
 // Bound by load and shared-memory latency: 2^22 samples 43 us (52 with 32 threads, staged loads
 // and seven crossings); 14 or 16 CTAs per SM with one buffer measured the same.
-__global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *__restrict__ E, int64_t e0, int64_t i0, int64_t o0,
+__global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *E, int64_t e0, int64_t i0, int64_t o0,
                                                        int64_t no, int64_t start, int V,
                                                        const float2 *__restrict__ H, const float2 *__restrict__ tw,
                                                        const float2 *__restrict__ tw2, float2 *__restrict__ y,
@@ -234,7 +243,7 @@ __global__ void __launch_bounds__(KT, 12) kk_filter_kernel(const float2 *__restr
   asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
   const float2 *src = E + (lo - e0) + t;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) x[q] = src[KT * q];
+  for (int q = 0; q < 16; ++q) x[q] = kk_load_behind_wait(src + KT * q);
   if (field) {
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
