@@ -347,6 +347,15 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 __device__ __forceinline__ void tc_grid_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_grid_trigger() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
+// A load of what the kernel directly in front writes: coherent, and kept behind the wait (__ldg
+// would take it for read-only data of the whole kernel, whose life begins while that kernel
+// still writes).  What was complete before the kernel in front started may go through __ldg.
+__device__ __forceinline__ uint2 tc_load_behind_wait(const uint2 *p) {
+  uint2 v;
+  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
+}
+
 __device__ __forceinline__ void tc_ld32(unsigned taddr, float (&v)[32]) {
   unsigned r[32];
   asm volatile(
@@ -570,7 +579,7 @@ __global__ void __launch_bounds__(TC_M) edge_in_kernel(const __grid_constant__ C
       const __nv_bfloat162 v0 = __floats2bfloat162_rn(p0.x, p0.y), v1 = __floats2bfloat162_rn(p1.x, p1.y);
       return make_uint2(*reinterpret_cast<const unsigned *>(&v0), *reinterpret_cast<const unsigned *>(&v1));
     } else {
-      return __ldg(reinterpret_cast<const uint2 *>(a.in + n * FEATP));
+      return tc_load_behind_wait(reinterpret_cast<const uint2 *>(a.in + n * FEATP));
     }
   };
   int it = 0;

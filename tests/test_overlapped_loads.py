@@ -27,7 +27,8 @@ def _kernel(path, name):
 
 
 # kernel, what it reads that the kernel in front of it writes: pointer, and how it is loaded
-CASES = [("kk.cu", "kk_filter_kernel", "E", r"kk_load_behind_wait\(src \+")]
+CASES = [("kk.cu", "kk_filter_kernel", "E", r"kk_load_behind_wait\(src \+"),
+         ("cnn.cu", "edge_in_kernel", "a.in", r"tc_load_behind_wait\([^;]*a\.in \+")]
 
 
 @pytest.mark.parametrize("path,name,pointer,load", CASES)
@@ -41,7 +42,7 @@ def test_reads_of_the_kernel_in_front(path, name, pointer, load):
     assert re.search(load, body[wait:]) and not re.search(load, body[:wait])
 
 
-@pytest.mark.parametrize("path,helper", [("kk.cu", "kk_load_behind_wait")])
+@pytest.mark.parametrize("path,helper", [("kk.cu", "kk_load_behind_wait"), ("cnn.cu", "tc_load_behind_wait")])
 def test_the_load_is_volatile_and_clobbers_memory(path, helper):
     text = open(os.path.join(CSRC, path)).read()
     m = re.search(helper + r"\([^)]*\)\s*\{(.*?)\n\}", text, flags=re.S)
