@@ -379,19 +379,22 @@ __global__ void __launch_bounds__(WBLOCK) wl4_kernel(const float4 *__restrict__ 
   const int64_t base = s0 - Wp;          // symbol of the lockstep's first step
   const int64_t p0 = base > 0 ? base : 0;
   const int64_t b_first = s_begin + (int64_t)blockIdx.x * WSEG4 * S - Wp;   // base of the warp's segment 0
-  const int64_t span = (int64_t)Wp + S;
-  const int64_t nch = (span + WCH - 1) / WCH;
+  // Chunks from the first that reaches a segment's start to the last before a segment's end:
+  // what the buffer holds, not W + S, which a caller may set far above it (40 symbols at
+  // S = 2^16: 14 us; all of W + S 419, S = 2^20 93 ms).
+  const int c_first = (int)(__reduce_min_sync(0xffffffffu, live ? (unsigned)(p0 - base) : ~0u) / WCH);
+  const int c_end = (int)((__reduce_max_sync(0xffffffffu, live ? (unsigned)(s1 - base) : 0u) + (WCH - 1)) / WCH);
   // chunk c of every segment: pairs base + c WCH + lane; zero outside the buffer or past the last segment
-  auto issue = [&](int64_t c) {
+  auto issue = [&](int c) {
 #pragma unroll
     for (int q = 0; q < WSEG4; ++q) {
-      const int64_t idx = b_first + (int64_t)q * S + c * WCH + lane;
+      const int64_t idx = b_first + (int64_t)q * S + (int64_t)c * WCH + lane;
       const bool ok = blockIdx.x * WSEG4 + q < nseg && idx >= 0 && idx < K;
       wl_cp16(&ring[c & 1][q][lane], ok ? (const void *)(x4 + idx) : (const void *)x4, ok ? 16 : 0);
     }
     wl_cp_commit();
   };
-  issue(0);
+  issue(c_first);
   WlRec4<MB> st;
   st.a0 = taps_in->m[half][2 * comp];
   st.a1 = taps_in->m[half][2 * comp + 1];
@@ -404,8 +407,8 @@ __global__ void __launch_bounds__(WBLOCK) wl4_kernel(const float4 *__restrict__ 
     st.ua = half ? make_float2(h.x, h.y) : make_float2(h.z, h.w);
   }
   const float mu_s = 2.f * mu;
-  for (int64_t c = 0; c < nch; ++c) {
-    if (c + 1 < nch) {
+  for (int c = c_first; c < c_end; ++c) {
+    if (c + 1 < c_end) {
       issue(c + 1);
       wl_cp_wait<1>();
     } else {
@@ -415,7 +418,7 @@ __global__ void __launch_bounds__(WBLOCK) wl4_kernel(const float4 *__restrict__ 
     const float2 *row = reinterpret_cast<const float2 *>(&ring[c & 1][seg][0]) + (1 - half);
 #pragma unroll 1
     for (int h = 0; h < WCH / WSUB; ++h) {
-      const int64_t t0 = c * WCH + h * WSUB;               // the same for every segment
+      const int64_t t0 = (int64_t)c * WCH + h * WSUB;      // the same for every segment
       const int64_t start = base + t0;
       const float2 *r = row + 2 * h * WSUB;
       const bool out = t0 >= Wp;                           // Wp is a multiple of 16
@@ -424,7 +427,7 @@ __global__ void __launch_bounds__(WBLOCK) wl4_kernel(const float4 *__restrict__ 
 #pragma unroll
       for (int t = 0; t < WPS; ++t) w[t] = 0u;
       float *zo = HAS_Z ? reinterpret_cast<float *>(z + start) + comp : nullptr;
-      if (t0 >= span || !__any_sync(0xffffffffu, live && start < s1)) break;
+      if (!__any_sync(0xffffffffu, live && start + WSUB > p0 && start < s1)) continue;
       if (__all_sync(0xffffffffu, whole)) {
         st.template steps<WSUB>(r, mu_s, [&](int q, float zv, bool neg, bool outer) {
           if (neg) w[(q * MB) >> 5] |= 1u << ((q * MB) & 31);
