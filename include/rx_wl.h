@@ -50,6 +50,8 @@ rx_status rx_wl_create(rx_wl **out, int mod_bits, int ntaps, int64_t max_symbols
 
 rx_status rx_wl_set_param(rx_wl *w, int key, double value);
 rx_status rx_wl_get_param(rx_wl *w, int key, double *value);
+/* Binds a stream.  After rx_wl_reset its work comes behind the reset, whichever stream
+ * that was enqueued on; otherwise the caller orders the streams. */
 rx_status rx_wl_set_cuda_stream(rx_wl *w, void *cuda_stream);
 
 /* Start taps (host array of 4 T floats: h[0..T) then g[0..T), each re, im).

@@ -183,4 +183,33 @@ cudaError_t launch_slide(const SlideArgs &a, cudaStream_t s);
 cudaError_t launch_cols_to_f32(float2 *dst, int64_t dst_stride, const void *src, int64_t src_stride, int64_t n,
                                int fmt, cudaStream_t s);
 
+// Where a reset left the stream that was bound then: work on a stream bound later comes
+// behind it.  The order is an event on the device, so that neither the host waits nor the
+// earlier stream is touched again (its owner may have destroyed it).
+struct ResetMark {
+  cudaEvent_t ev = nullptr;
+  bool set = false;
+  cudaError_t create() { return cudaEventCreateWithFlags(&ev, cudaEventDisableTiming); }
+  void destroy() {
+    if (ev) cudaEventDestroy(ev);
+    ev = nullptr;
+    set = false;
+  }
+  // after the reset's work on s; inside a capture the graph's launch orders it
+  cudaError_t record(cudaStream_t s) {
+    cudaStreamCaptureStatus cap;
+    cudaError_t e = cudaStreamIsCapturing(s, &cap);
+    set = e == cudaSuccess && cap == cudaStreamCaptureStatusNone;
+    return set ? cudaEventRecord(ev, s) : e;
+  }
+  cudaError_t bind(cudaStream_t next) {
+    if (!set) return cudaSuccess;
+    cudaStreamCaptureStatus cap;
+    const cudaError_t e = cudaStreamIsCapturing(next, &cap);
+    if (e != cudaSuccess) return e;
+    // an event from outside a capture is waited for by a node of the graph
+    return cudaStreamWaitEvent(next, ev, cap == cudaStreamCaptureStatusNone ? 0 : cudaEventWaitExternal);
+  }
+};
+
 }  // namespace rx

@@ -528,7 +528,7 @@ struct rx_wl {
   WlTaps start{};            // host copy of the start taps (matrix form)
   WlTaps *dev = nullptr;     // [0], [1]: wave-start taps ping-pong; [2]: acquisition end
   float4 *tail = nullptr;    // [2] the previous buffer's last two samples (zero for the first), by `cur`
-  bool start_pending = false;   // a reset's start state may still be on its way
+  ResetMark mark;               // a reset's start state may still be on its way
   int cur = 0;               // which of dev[0..1] holds the taps for the next call
   cudaStream_t stream = nullptr;
   bool profile = false;
@@ -570,9 +570,9 @@ void from_matrix(const WlTaps &o, double *t) {
 rx_status upload_start(rx_wl *w, bool wait) {
   wl_start_kernel<<<1, 1, 0, w->stream>>>(w->dev, w->start, w->tail);
   cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && wait) e = cudaStreamSynchronize(w->stream);
+  if (e == cudaSuccess) e = wait ? cudaStreamSynchronize(w->stream) : w->mark.record(w->stream);
   if (e != cudaSuccess) return wfail(w, RX_ECUDA, std::string("start taps: ") + cudaGetErrorString(e));
-  w->start_pending = !wait;
+  if (wait) w->mark.set = false;
   w->cur = 0;
   return RX_OK;
 }
@@ -602,13 +602,16 @@ rx_status rx_wl_create(rx_wl **out, int mod_bits, int ntaps, int64_t max_symbols
   double t[4 * WT] = {0};
   t[2 * WC] = 1.0;
   w->start = to_matrix(t);
-  if (cudaMalloc(&w->dev, 3 * sizeof(WlTaps)) != cudaSuccess || cudaMalloc(&w->tail, 2 * sizeof(float4)) != cudaSuccess) {
+  if (w->mark.create() != cudaSuccess || cudaMalloc(&w->dev, 3 * sizeof(WlTaps)) != cudaSuccess ||
+      cudaMalloc(&w->tail, 2 * sizeof(float4)) != cudaSuccess) {
     cudaGetLastError();
+    w->mark.destroy();
     cudaFree(w->dev);
     delete w;
     return RX_ENOMEM;
   }
   if (upload_start(w, true) != RX_OK) {
+    w->mark.destroy();
     cudaFree(w->dev);
     cudaFree(w->tail);
     delete w;
@@ -662,11 +665,9 @@ rx_status rx_wl_get_param(rx_wl *w, int key, double *v) {
 
 rx_status rx_wl_set_cuda_stream(rx_wl *w, void *s) {
   if (!w) return RX_EINVAL;
-  // a reset's start state on the old stream comes before work on the new one
-  if (w->start_pending && (cudaStream_t)s != w->stream) {
-    const cudaError_t e = cudaStreamSynchronize(w->stream);
+  if ((cudaStream_t)s != w->stream) {
+    const cudaError_t e = w->mark.bind((cudaStream_t)s);
     if (e != cudaSuccess) return wfail(w, RX_ECUDA, std::string("stream change: ") + cudaGetErrorString(e));
-    w->start_pending = false;
   }
   w->stream = (cudaStream_t)s;
   return RX_OK;
@@ -772,6 +773,7 @@ void rx_wl_destroy(rx_wl *w) {
   if (!w) return;
   cudaStreamSynchronize(w->stream);
   drop_events(w);
+  w->mark.destroy();
   cudaFree(w->dev);
   cudaFree(w->tail);
   delete w;
