@@ -183,7 +183,9 @@ rx_status rx_create(rx_stream **out, double baud, int sps, double L_km,
 rx_status rx_set_param(rx_stream *rx, int key, double value);
 rx_status rx_get_param(rx_stream *rx, int key, double *value);
 
-/* Bind a CUDA stream (a cudaStream_t, e.g. torch.cuda.Stream.cuda_stream). */
+/* Bind a CUDA stream (a cudaStream_t, e.g. torch.cuda.Stream.cuda_stream).  After
+ * rx_reset its work comes behind the reset, whichever stream that was enqueued on;
+ * within a recording the caller orders the streams. */
 rx_status rx_set_cuda_stream(rx_stream *rx, void *cuda_stream);
 
 /* Allocate all device state for calls of up to max_call_samples sample-times.

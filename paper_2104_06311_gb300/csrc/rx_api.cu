@@ -99,6 +99,7 @@ struct rx_stream {
   int pieces = 12;                  // pipeline pieces per call (RX_P_PIPELINE)
   bool pieces_set = false;          // chosen by the caller: else at most `pieces` (auto_pieces)
   cudaStream_t sub[3] = {nullptr, nullptr, nullptr};   // CDC, equaliser, BPS streams
+  ResetMark mark;                   // a reset's start state may still be on its way
   cudaEvent_t ev_fork = nullptr;
   cudaEvent_t ev_piece[3][kMaxPieces] = {};
   // ---- per-stage measurement (CUDA events on the bound stream)
@@ -204,6 +205,7 @@ void release(rx_stream *rx) {
     if (rx->sub[i]) cudaStreamDestroy(rx->sub[i]), rx->sub[i] = nullptr;
   }
   if (rx->ev_fork) cudaEventDestroy(rx->ev_fork), rx->ev_fork = nullptr;
+  rx->mark.destroy();
   rx->ev_pool.clear();
   rx->ev_pending.clear();
   rx->ev_used = 0;
@@ -521,6 +523,7 @@ rx_status rx_get_param(rx_stream *rx, int key, double *v) {
 
 rx_status rx_set_cuda_stream(rx_stream *rx, void *s) {
   if (!rx) return RX_EINVAL;
+  if (rx->reserved && (cudaStream_t)s != rx->stream) RX_CUDA(rx->mark.bind((cudaStream_t)s), "stream change");
   rx->stream = (cudaStream_t)s;
   return RX_OK;
 }
@@ -583,6 +586,7 @@ rx_status rx_reserve(rx_stream *rx, int64_t max_call) {
       e = cudaEventCreateWithFlags(&rx->ev_piece[i][j], cudaEventDisableTiming);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&rx->ev_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = rx->mark.create();
   if (e != cudaSuccess) { release(rx); return cuda_fail(rx, e, "pipeline streams"); }
   e = launch_tables(rx->H, rx->tw, rx->N, rx->baud, rx->L_km, rx->D, rx->lam_nm, rx->rolloff, rx->stream);
   if (e != cudaSuccess) { release(rx); return cuda_fail(rx, e, "filter tables"); }
@@ -613,8 +617,9 @@ rx_status rx_reset(rx_stream *rx) {
   reset_host_state(rx);
   if (!rx->reserved) return RX_OK;
   rx_status s = init_device_state(rx);
-  if (s != RX_OK) return s;
-  return post_error_copy(rx);
+  if (s == RX_OK) s = post_error_copy(rx);
+  if (s == RX_OK) RX_CUDA(rx->mark.record(rx->stream), "reset");
+  return s;
 }
 
 rx_status rx_sync(rx_stream *rx) {

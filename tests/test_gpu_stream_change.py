@@ -45,3 +45,45 @@ def test_widely_linear():
     assert busy and took < 0.05, (busy, took)
     assert torch.equal(got, want) and torch.equal(got_z, want_z)
     eq.close()
+
+
+@pytest.mark.parametrize("chunk", [None, 60_000])
+def test_receiver(chunk):
+    import torch
+    import linksim as L
+    from chain_helpers import make_receiver, rx_params
+    lk = L.Link(n_sym=60_000, L_km=500.0, snr_db=12.0, seed=2104063181)
+    g = L.generate(lk)
+    rx = make_receiver(rx_params(lk, g.in_scale), SYM_OUT=1)
+    x = torch.from_numpy(g.samples).cuda()
+    rx.reserve(x.shape[0])
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+
+    def calls():
+        out = rx.alloc_out(lk.n_sym + 64, sym=True)
+        pos = 0
+        step = chunk or x.shape[0]
+        for a in list(range(0, x.shape[0], step)) + [None]:
+            _, n, _, _ = rx.process(None if a is None else x[a:a + step], out, sym_offset=pos)
+            pos += n
+        return out, pos
+
+    rx.set_cuda_stream(s1)
+    with torch.cuda.stream(s1):
+        want, n = calls()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s1):
+        torch.cuda._sleep(BUSY)
+        rx.reset()
+    t0 = time.perf_counter()
+    rx.set_cuda_stream(s2)
+    took = time.perf_counter() - t0
+    busy = not s1.query()
+    with torch.cuda.stream(s2):
+        got, m = calls()
+    torch.cuda.synchronize()
+    assert busy and took < 0.05, (busy, took)
+    assert m == n == lk.n_sym
+    assert torch.equal(got["bits"], want["bits"]) and torch.equal(got["sym"][:, :n], want["sym"][:, :n])
+    rx.close()
