@@ -465,7 +465,7 @@ rx_status enqueue(rx_batch *b, const rx_in *ins, rx_out *outs, cudaStream_t s, b
     B.bhat = c.bh;
     B.bh_base = 0;
     B.bh_stride = c.y_stride;
-    B.chunk = c.C;
+    B.chunk = B.grid = c.C;
     B.n_chunks = (K + c.C - 1) / c.C;
     B.chunk_r = c.chunk_r;
     B.chunk_s2 = c.chunk_s2;

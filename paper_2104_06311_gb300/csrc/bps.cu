@@ -78,8 +78,15 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_slide(BpsLaunch L) {
     if (edge && (i < v_lo || i >= v_hi)) return 0.f;
     return qam_dist<MB>(cmul(ys[i], rot));
   };
-  for (int i = 0; i < M; ++i) ring[i * 32 + lane] = dist(i);   // window of symbol `start`
-  int s_out = 0;                                 // slot of the oldest symbol in the window
+  // window of symbol `start`.  The re-sum below adds the ring by slots, so the order of a sum
+  // is that of a chunk begun at the last grid point, whatever the length of this one: a near
+  // tie falls the same way however a recording is cut into calls, pieces and chunks
+  const int o = (int)((a - L.k_lo) % L.grid) % M;
+  for (int i = 0; i < M; ++i) {
+    const int q = o + i;
+    ring[(q < M ? q : q - M) * 32 + lane] = dist(i);
+  }
+  int s_out = o;                                 // slot of the oldest symbol in the window
   float D = 0.f;
   int prev = 0, R = 0;
   float s2 = 0.f;

@@ -111,7 +111,7 @@ extern "C" rx_status rx_bps_demap_noalloc(const float *y, int64_t y_stride, int6
   B.bhat = reinterpret_cast<int8_t *>(base + kOffBhat);
   B.bh_base = 0;
   B.bh_stride = kNoAllocMaxSymbols;
-  B.chunk = kNoAllocChunk;
+  B.chunk = B.grid = kNoAllocChunk;
   B.n_chunks = (n_symbols + kNoAllocChunk - 1) / kNoAllocChunk;
   B.chunk_m = reinterpret_cast<int64_t *>(base + kOffChunkM);
   B.chunk_r = reinterpret_cast<int *>(base + kOffChunkR);

@@ -864,6 +864,7 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       B.bh_base = rx->y_base;
       B.bh_stride = rx->y_cap;
       B.chunk = bps_chunk(rx, kj - kdone);
+      B.grid = rx->C;
       B.n_chunks = (kj - kdone + B.chunk - 1) / B.chunk;
       if (B.n_chunks > rx->chunk_cap) return fail(rx, RX_EINVAL, "chunk table overflow");
       B.chunk_r = rx->chunk_r;

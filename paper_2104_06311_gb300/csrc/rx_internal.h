@@ -118,6 +118,8 @@ struct BpsLaunch {
   int64_t K_end;            // symbols known to exist (stream end if flushed)
   int64_t A, span;          // region layout
   int chunk;                // chunk length (symbols)
+  int grid;                 // a multiple of chunk that regions start on: the sliding pass adds its
+                            // window in an order that depends on the position on this grid alone
   int64_t n_chunks;
   int Nb, mod_bits;
   int need_s2;              // 1: sum |z - dec z|^2 per chunk (only the LLRs use sigma^2)

@@ -39,3 +39,25 @@ def test_pieces_and_chunks(mod, nb):
         assert np.array_equal(a["sym"][:, :K], b["sym"][:, :K])
         la, lb = a["llr"][:, :K * m], b["llr"][:, :K * m]
         assert np.max(np.abs(la - lb) / (np.abs(la) + 1e-30)) <= (2 * 256 + 4) * 2.0 ** -24
+
+
+@pytest.mark.parametrize("mod,nb,seed", [("16qam", 7, 1), ("16qam", 24, 2), ("qpsk", 7, 3), ("qpsk", 50, 4), ("16qam", 41, 5),
+                                         ("qpsk", 0, 6), ("16qam", 32, 7)])
+def test_near_ties_fall_alike(mod, nb, seed):
+    # half windows of the sliding pass (and one of the register blocks), at a noise that makes
+    # near ties of two angles common: every angle the same, so every symbol
+    import torch
+    lk = L.Link(mod=mod, n_sym=600_000, L_km=200.0, snr_db=11.0 if mod == "qpsk" else 17.0, seed=2104063190 + seed)
+    g = L.generate(lk)
+    p = rx_params(lk, g.in_scale, fo_track=mod == "qpsk")
+    x = torch.from_numpy(g.samples).cuda()
+    want = None
+    for chunk, kw in ((None, dict(PIPELINE=1)), (None, {}), (None, dict(PIPELINE=12)), (150_000, {}), (400_002, {})):
+        rx = make_receiver(p, SYM_OUT=1, BPS_HALFWIN=nb, **kw)
+        o = rx.run_stream(x, chunk=chunk, sym=True)
+        got = (o["bits"].cpu().numpy(), o["sym"][:, :o["n"]].cpu().numpy())
+        rx.close()
+        if want is None:
+            want = got
+        assert np.array_equal(got[1], want[1]), (chunk, kw, int((got[1] != want[1]).sum()))
+        assert np.array_equal(got[0], want[0])
