@@ -66,7 +66,7 @@ struct Chan {
   float2 *H = nullptr, *tw = nullptr, *u = nullptr, *y = nullptr, *tap_slot = nullptr;
   int8_t *bh = nullptr;
   int *chunk_r = nullptr;
-  float *chunk_s2 = nullptr;
+  float *part_s2 = nullptr;
   int64_t *chunk_m = nullptr;
   double *region_s2 = nullptr;
   EqState *st = nullptr;
@@ -466,9 +466,10 @@ rx_status enqueue(rx_batch *b, const rx_in *ins, rx_out *outs, cudaStream_t s, b
     B.bh_base = 0;
     B.bh_stride = c.y_stride;
     B.chunk = B.grid = c.C;
+    B.part = bps_part(c.C);
     B.n_chunks = (K + c.C - 1) / c.C;
     B.chunk_r = c.chunk_r;
-    B.chunk_s2 = c.chunk_s2;
+    B.part_s2 = c.part_s2;
     B.chunk_m = c.chunk_m;
     B.m_carry = b->m_carry + 2 * i;
     B.region_s2 = c.region_s2;
@@ -620,7 +621,7 @@ rx_status rx_batch_create(rx_batch **out, int n_ch, const rx_chan_cfg *cfgs) {
     BX_ALLOC(c.y, (size_t)2 * c.y_stride);
     BX_ALLOC(c.bh, (size_t)2 * c.y_stride);
     BX_ALLOC(c.chunk_r, (size_t)2 * c.chunk_cap);
-    BX_ALLOC(c.chunk_s2, (size_t)2 * c.chunk_cap);
+    BX_ALLOC(c.part_s2, (size_t)2 * (bps_part_row(c.K_cap, bps_part(c.C)) + 4));
     BX_ALLOC(c.chunk_m, (size_t)2 * c.chunk_cap);
     BX_ALLOC(c.region_s2, (size_t)2 * c.region_cap);
     BX_ALLOC(c.st, 1);

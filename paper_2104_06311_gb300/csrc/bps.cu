@@ -12,7 +12,8 @@
 //   m_k = m_{k-1} + r_k,  z_k = y_k e^{-j phi_bhat} (-j)^{m_k}.
 // Pass 1: one warp per chunk [a, b) of symbols, lane = test angle; argmin by a
 //   warp min-reduction on the float bits plus a ballot; writes bhat (int8), the
-//   chunk's sum of r_k over a < k < b and of |z - dec z|^2 = d_{k,bhat}.  With
+//   chunk's sum of r_k over a < k < b and, for the LLRs, sums of
+//   |z - dec z|^2 = d_{k,bhat} over 64 symbols each.  With
 //   the default half window (Nb = 16, a 33-symbol window) the window sums come
 //   from two 32-symbol blocks of distances in registers (pass1_blocks); other
 //   half windows slide a ring of distances in shared memory.
@@ -37,6 +38,10 @@ __device__ __forceinline__ int unwrap_step(int prev, int cur) {
 }
 
 __device__ __forceinline__ int64_t chunk_lo(const BpsLaunch &L, int64_t j) { return L.k_lo + j * L.chunk; }
+// the partial sums of polarisation p from symbol k on
+__device__ __forceinline__ float *part_sums(const BpsLaunch &L, int p, int64_t k) {
+  return L.part_s2 + p * bps_part_row(L.k_hi - L.k_lo, L.part) + (k - L.k_lo) / L.part;
+}
 }  // namespace
 
 // Per-warp shared memory of pass 1: the d ring (M x 32 floats), the staged
@@ -90,6 +95,7 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_slide(BpsLaunch L) {
   float D = 0.f;
   int prev = 0, R = 0;
   float s2 = 0.f;
+  float *parts = NEED_S2 ? part_sums(L, p, a) : nullptr;
   const int nt = (int)(b - start);
   // kGroup symbols at a time: first their window sums (a sliding chain per lane),
   // then their independent warp argmins back to back, then the unwrap in order
@@ -138,14 +144,16 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_slide(BpsLaunch L) {
         prev = bs;
       }
     }
+    if (NEED_S2 && (((t0 + kGroup) & (L.part - 1)) == 0 || t0 + kGroup >= nt)) {
+      if (lane == 0) *parts = s2;
+      ++parts;
+      s2 = 0.f;
+    }
   }
   __syncwarp();
   int8_t *bh = L.bhat + (int64_t)p * L.bh_stride - L.bh_base;
   for (int i = lane; i < (int)(b - a); i += 32) bh[a + i] = bq[i];
-  if (lane == 0) {
-    L.chunk_r[(int64_t)p * L.n_chunks + j] = R;
-    L.chunk_s2[(int64_t)p * L.n_chunks + j] = s2;
-  }
+  if (lane == 0) L.chunk_r[(int64_t)p * L.n_chunks + j] = R;
 }
 
 // Pass 1 at half windows Nb = 16 M (M = 1..4): the (32 M + 1)-symbol window of
@@ -171,8 +179,8 @@ __host__ __device__ inline size_t pass1_blk_warp_bytes(int chunk, int Nb) {
 }
 
 template <int MB, bool NEED_S2, bool EDGE, int M>
-__device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_hi, float2 rot, int nt, int lane,
-                                             int8_t *bq, unsigned *ties, int &R, float &s2) {
+__device__ __forceinline__ void pass1_blocks(float2 *ys, int v_lo, int v_hi, float2 rot, int nt, int lane,
+                                             int8_t *bq, unsigned *ties, int &R, int part, float *parts) {
   constexpr unsigned FULL = 0xffffffffu;
   auto dist = [](float2 v, float2 ph) -> float {
     const float2 w = cmul(v, ph);
@@ -205,6 +213,7 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
     }
   }
   int prev = 0;
+  float s2 = 0.f;
   for (int base = 0; base < nt; base += 32) {
     const float2 *yb = ys + base;
     const int cnt = min(32, nt - base);          // symbols of this block
@@ -240,6 +249,11 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
       const float2 rb = make_float2(__shfl_sync(FULL, rot.x, mybs), __shfl_sync(FULL, rot.y, mybs));
       const float own = dist(yb[lane + 16 * M], rb);
       s2 += lane < cnt ? own : 0.f;
+      // a part's lane sums wait in its first positions, which no later block reads
+      if (((base + 32) & (part - 1)) == 0 || base + 32 >= nt) {
+        reinterpret_cast<float *>(ys + base / part * part)[lane] = s2;
+        s2 = 0.f;
+      }
     }
     // unwrap steps of the block's symbols at once (r of the chunk's first symbol: the scan)
     const int up = __shfl_up_sync(FULL, mybs, 1);
@@ -261,10 +275,17 @@ __device__ __forceinline__ void pass1_blocks(const float2 *ys, int v_lo, int v_h
       T[M - 2] = t;
     }
   }
-  if (NEED_S2) {
+  if (NEED_S2) {   // eight lanes add a part's sums (a chunk has at most four parts)
+    __syncwarp();
+    const int q = lane >> 3;
+    float s = 0.f;
+    if (q * part < nt) {
+      const float2 *v = ys + q * part + 2 * (lane & 7);
+      s = (v[0].x + v[0].y) + (v[1].x + v[1].y);
+    }
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) s2 += __shfl_xor_sync(FULL, s2, o);
-    if (MB == 4) s2 *= 0.1f;
+    for (int o = 4; o >= 1; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
+    if ((lane & 7) == 0 && q * part < nt) parts[q] = MB == 4 ? s * 0.1f : s;
   }
 }
 
@@ -298,28 +319,31 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_blk(BpsLaunch L) {
   __syncwarp();
   const int64_t v_lo = -lo, v_hi = L.K_end - lo;  // valid staged positions [v_lo, v_hi)
   int R = 0;
-  float s2 = 0.f;
+  float *const parts = NEED_S2 ? part_sums(L, p, a) : nullptr;
   if (v_lo > 0 || v_hi < n_ys) {                  // the window touches a stream end
     pass1_blocks<MB, NEED_S2, true, M>(ys, (int)max(v_lo, (int64_t)0), (int)min(v_hi, (int64_t)n_ys), rot, nt, lane,
-                                       bq, ties, R, s2);
+                                       bq, ties, R, L.part, parts);
   } else {
-    pass1_blocks<MB, NEED_S2, false, M>(ys, 0, n_ys, rot, nt, lane, bq, ties, R, s2);
+    pass1_blocks<MB, NEED_S2, false, M>(ys, 0, n_ys, rot, nt, lane, bq, ties, R, L.part, parts);
   }
   __syncwarp();
   int8_t *bh = L.bhat + (int64_t)p * L.bh_stride - L.bh_base;
   for (int i = lane; i < nt; i += 32) bh[a + i] = bq[i];
-  if (lane == 0) {
-    L.chunk_r[(int64_t)p * L.n_chunks + j] = R;
-    L.chunk_s2[(int64_t)p * L.n_chunks + j] = s2;
-  }
+  if (lane == 0) L.chunk_r[(int64_t)p * L.n_chunks + j] = R;
 }
 
 // One CTA per pol.  A thread owns a run of chunks; the prefix over the 1024 threads goes
 // by warp shuffles and one pass over the 32 warp totals.  A region's noise variance is a
-// warp's sum over its chunks (lane-strided in double, then a butterfly).  Bound by the
-// latency of its loads; region sums by one thread each took 17.5 us of a call's tail at 128
-// chunks per region, the warps take 10 at 512.
-__global__ void __launch_bounds__(1024) bps_scan(BpsLaunch L) {
+// warp's sum over its partial sums (lane-strided in double, then a butterfly), the same
+// whatever the launch's range and chunks.  Bound by the latency of its loads; region sums by
+// one thread each took 17.5 us of a call's tail at 128 sums per region, the warps take 10 at
+// 512.  Without LLRs (NEED_S2 false) it keeps to 32 registers, some words spilled: with more a
+// CTA waits longer for room beside the other kernels of a batch (64 channels, 56 registers:
+// 6166 -> 6194 us).  The
+// regions take up to 64: 2^20 16QAM symbols with LLRs 993 us either way, 700,001 with FP16 LLRs
+// 745 us at 32 and a few words spilled, 743 at 64, six channels 389 and 387.
+template <bool NEED_S2>
+__global__ void __launch_bounds__(1024, NEED_S2 ? 1 : 2) bps_scan(BpsLaunch L) {
   __shared__ int64_t part[32];
   const int p = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int64_t n = L.n_chunks;
@@ -356,19 +380,28 @@ __global__ void __launch_bounds__(1024) bps_scan(BpsLaunch L) {
     run += L.chunk_r[(int64_t)p * n + c];
   }
   if (t == 0) L.m_carry[p] = carry + total;      // every thread read it before the barrier
-  if (!L.need_s2) return;   // sigma^2 feeds the LLRs only
+  if (!NEED_S2) return;     // sigma^2 feeds the LLRs only
   // regions: [0, A), then [A + r span, ...), clipped to [k_lo, k_hi) (calls emit whole
   // regions, so a region's chunks start at its first symbol)
   const int64_t r_lo = L.k_lo < L.A ? 0 : 1 + (L.k_lo - L.A) / L.span;
   const int64_t r_hi = L.k_hi <= L.A ? 1 : 1 + (L.k_hi - 1 - L.A) / L.span + 1;
+  const bool rows = L.grid % (4 * L.part) == 0;
   for (int64_t r = r_lo + warp; r < r_hi; r += 32) {
     const int64_t s_r = r == 0 ? 0 : L.A + (r - 1) * L.span;
     const int64_t e_r = min(r == 0 ? L.A : s_r + L.span, L.k_hi);
-    const int64_t q0 = (s_r - L.k_lo) / L.chunk;
-    const int64_t q1 = min(n, (e_r - L.k_lo + L.chunk - 1) / L.chunk);   // chunks starting before e_r
+    const float *parts = part_sums(L, p, s_r);             // (regions start on a part)
+    const int64_t np = bps_parts(e_r - s_r, L.part);
     double acc = 0.0;
-#pragma unroll 4
-    for (int64_t c = q0 + lane; c < q1; c += 32) acc += (double)L.chunk_s2[(int64_t)p * n + c];
+#pragma unroll 2
+    for (int64_t c = 4 * lane; c < np; c += 128) {
+      // four sums at a time in FP32: the FP64 unit is narrow (each of them in FP64: 1005 us for
+      // the 2^20 symbols)
+      const int64_t m = np - c;                            // sums that are there
+      float4 v;
+      if (rows) v = *reinterpret_cast<const float4 *>(parts + c);
+      else v = make_float4(parts[c], m > 1 ? parts[c + 1] : 0.f, m > 2 ? parts[c + 2] : 0.f, m > 3 ? parts[c + 3] : 0.f);
+      acc += (double)((v.x + (m > 1 ? v.y : 0.f)) + ((m > 2 ? v.z : 0.f) + (m > 3 ? v.w : 0.f)));
+    }
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     // 1 / sigma^2, what the demapping multiplies by
@@ -537,7 +570,8 @@ cudaError_t launch_bps(const BpsLaunch &L, cudaStream_t s) {
 #undef RX_BLK_M
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  bps_scan<<<2, 1024, 0, s>>>(L);
+  if (L.need_s2) bps_scan<true><<<2, 1024, 0, s>>>(L);
+  else bps_scan<false><<<2, 1024, 0, s>>>(L);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (L.mod_bits == 4) {

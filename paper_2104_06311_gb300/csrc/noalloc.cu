@@ -37,8 +37,7 @@ constexpr int64_t kNoAllocChunks = kNoAllocMaxSymbols / kNoAllocChunk;
 constexpr size_t kOffBhat = 0;                                              // int8 [2][max]
 constexpr size_t kOffChunkM = kOffBhat + 2 * kNoAllocMaxSymbols;            // int64 [2][chunks]
 constexpr size_t kOffChunkR = kOffChunkM + 2 * kNoAllocChunks * 8;          // int32 [2][chunks]
-constexpr size_t kOffChunkS2 = kOffChunkR + 2 * kNoAllocChunks * 4;         // float [2][chunks]
-constexpr size_t kOffCarry = kOffChunkS2 + 2 * kNoAllocChunks * 4;          // int64 [2]
+constexpr size_t kOffCarry = kOffChunkR + 2 * kNoAllocChunks * 4;           // int64 [2]
 constexpr size_t kOffRegion = kOffCarry + 256;                              // double [2]
 constexpr size_t kScratchBytes = kOffRegion + 256;
 
@@ -112,10 +111,10 @@ extern "C" rx_status rx_bps_demap_noalloc(const float *y, int64_t y_stride, int6
   B.bh_base = 0;
   B.bh_stride = kNoAllocMaxSymbols;
   B.chunk = B.grid = kNoAllocChunk;
+  B.part = bps_part(kNoAllocChunk);
   B.n_chunks = (n_symbols + kNoAllocChunk - 1) / kNoAllocChunk;
   B.chunk_m = reinterpret_cast<int64_t *>(base + kOffChunkM);
   B.chunk_r = reinterpret_cast<int *>(base + kOffChunkR);
-  B.chunk_s2 = reinterpret_cast<float *>(base + kOffChunkS2);
   B.m_carry = reinterpret_cast<int64_t *>(base + kOffCarry);
   B.region_s2 = reinterpret_cast<double *>(base + kOffRegion);
   B.k_lo = 0;

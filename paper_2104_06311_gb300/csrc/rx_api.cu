@@ -83,9 +83,9 @@ struct rx_stream {
   bool bar_set = false;             // the set of the next equaliser launch (zero by then)
   int *err = nullptr;
   int *chunk_r = nullptr;
-  float *chunk_s2 = nullptr;
+  float *part_s2 = nullptr;
   int64_t *chunk_m = nullptr, *m_carry = nullptr;
-  int64_t chunk_cap = 0;
+  int64_t chunk_cap = 0, part_cap = 0;
   double *region_s2 = nullptr;
   int64_t region_cap = 0;
   unsigned *ber_counts = nullptr;
@@ -192,7 +192,7 @@ rx_status dalloc(rx_stream *rx, Tp **p, size_t count) {
 void release(rx_stream *rx) {
   void *ptrs[] = {rx->H, rx->tw, rx->tail[0], rx->tail[1], rx->u[0], rx->u[1], rx->y[0], rx->y[1],
                   rx->bh[0], rx->bh[1], rx->st, rx->fo_part, rx->tap_slot, rx->trace, rx->trace_fo,
-                  rx->inner, rx->barrier, rx->err, rx->chunk_r, rx->chunk_s2, rx->chunk_m, rx->m_carry,
+                  rx->inner, rx->barrier, rx->err, rx->chunk_r, rx->part_s2, rx->chunk_m, rx->m_carry,
                   rx->region_s2, rx->ber_counts, rx->ber_acc, rx->ber_sync};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -222,7 +222,7 @@ void release(rx_stream *rx) {
   rx->barrier = nullptr;
   rx->err = nullptr;
   rx->chunk_r = nullptr;
-  rx->chunk_s2 = nullptr;
+  rx->part_s2 = nullptr;
   rx->chunk_m = rx->m_carry = nullptr;
   rx->region_s2 = nullptr;
   rx->ber_counts = nullptr;
@@ -544,6 +544,7 @@ rx_status rx_reserve(rx_stream *rx, int64_t max_call) {
   rx->u_cap |= 1;
   rx->y_cap = max_call / 2 + 4 * region + 4 * rx->Nb + 4096;
   rx->chunk_cap = rx->y_cap / rx->C + 16 + kFineChunks;
+  rx->part_cap = bps_part_row(rx->y_cap, bps_part(rx->C));
   rx->region_cap = rx->y_cap / std::min(rx->A_full > 0 ? rx->A_full : rx->span, rx->span) + 16;
 #define RX_ALLOC(ptr, count)              \
   do {                                    \
@@ -567,7 +568,7 @@ rx_status rx_reserve(rx_stream *rx, int64_t max_call) {
   RX_ALLOC(rx->barrier, 2 * kEqBarrierWords);
   RX_ALLOC(rx->err, 1);
   RX_ALLOC(rx->chunk_r, (size_t)2 * rx->chunk_cap);
-  RX_ALLOC(rx->chunk_s2, (size_t)2 * rx->chunk_cap);
+  RX_ALLOC(rx->part_s2, (size_t)2 * rx->part_cap);
   RX_ALLOC(rx->chunk_m, (size_t)2 * rx->chunk_cap);
   RX_ALLOC(rx->m_carry, 2);
   RX_ALLOC(rx->region_s2, (size_t)2 * rx->region_cap);
@@ -865,10 +866,11 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       B.bh_stride = rx->y_cap;
       B.chunk = bps_chunk(rx, kj - kdone);
       B.grid = rx->C;
+      B.part = bps_part(rx->C);
       B.n_chunks = (kj - kdone + B.chunk - 1) / B.chunk;
-      if (B.n_chunks > rx->chunk_cap) return fail(rx, RX_EINVAL, "chunk table overflow");
+      if (B.n_chunks > rx->chunk_cap || bps_part_row(kj - kdone, B.part) > rx->part_cap) return fail(rx, RX_EINVAL, "chunk table overflow");
       B.chunk_r = rx->chunk_r;
-      B.chunk_s2 = rx->chunk_s2;
+      B.part_s2 = rx->part_s2;
       B.chunk_m = rx->chunk_m;
       B.m_carry = rx->m_carry;
       B.region_s2 = rx->region_s2;

@@ -110,7 +110,7 @@ struct BpsLaunch {
   const float2 *y; int64_t y_base, y_stride;
   int8_t *bhat; int64_t bh_base, bh_stride;
   int *chunk_r;             // [2][n_chunks] unwrap step sums
-  float *chunk_s2;          // [2][n_chunks] sum of |z - dec z|^2
+  float *part_s2;           // [2][bps_part_row] sums of |z - dec z|^2 over `part` symbols each (need_s2)
   int64_t *chunk_m;         // [2][n_chunks] exclusive prefix (filled by the scan)
   int64_t *m_carry;         // [2] unwrap count carried from earlier calls
   double *region_s2;        // [2][n_regions] 1 / sigma^2 of regions in this call
@@ -120,9 +120,12 @@ struct BpsLaunch {
   int chunk;                // chunk length (symbols)
   int grid;                 // a multiple of chunk that regions start on: the sliding pass adds its
                             // window in an order that depends on the position on this grid alone
+  int part;                 // 32 or 64, divides chunk: symbols of an FP32 partial sum of the noise
+                            // variance, the same for every chunk length, so that an LLR does not
+                            // depend on how the recording is cut
   int64_t n_chunks;
   int Nb, mod_bits;
-  int need_s2;              // 1: sum |z - dec z|^2 per chunk (only the LLRs use sigma^2)
+  int need_s2;              // 1: sum |z - dec z|^2 (only the LLRs use sigma^2)
   // outputs
   uint32_t *bits; int64_t bits_stride;
   float *llr; int64_t llr_stride;
@@ -130,6 +133,12 @@ struct BpsLaunch {
   float2 *sym; int64_t sym_stride;
   int64_t out_first;        // stream index of output symbol 0
 };
+
+// Symbols per partial sum for chunks of `chunk` symbols (a power of two >= 32), how many
+// partial sums n symbols have, and the row of them that a polarisation takes (whole fours).
+__host__ __device__ inline int bps_part(int chunk) { return chunk < 64 ? chunk : 64; }
+__host__ __device__ inline int64_t bps_parts(int64_t n, int part) { return (n + part - 1) / part; }
+__host__ __device__ inline int64_t bps_part_row(int64_t n, int part) { return (bps_parts(n, part) + 3) / 4 * 4; }
 
 // Launchers (defined in the .cu files).
 cudaError_t launch_tables(float2 *H, float2 *tw, int N, double baud, double L_km, double D,

@@ -61,3 +61,23 @@ def test_near_ties_fall_alike(mod, nb, seed):
             want = got
         assert np.array_equal(got[1], want[1]), (chunk, kw, int((got[1] != want[1]).sum()))
         assert np.array_equal(got[0], want[0])
+
+
+@pytest.mark.parametrize("mod,nb,form", [("qpsk", 16, 1), ("16qam", 64, 1), ("16qam", 16, 2), ("qpsk", 24, 1), ("16qam", 7, 1)])
+def test_llrs_do_not_depend_on_the_cut(mod, nb, form):
+    # the noise variance is summed over fixed spans of symbols, so the LLRs are the same to the
+    # last bit in one call, in any number of pieces and in calls
+    import torch
+    lk = L.Link(mod=mod, n_sym=600_000, L_km=300.0, snr_db=13.0 if mod == "qpsk" else 20.0, seed=2104063200 + nb)
+    g = L.generate(lk)
+    p = rx_params(lk, g.in_scale, fo_track=mod == "qpsk")
+    x = torch.from_numpy(g.samples).cuda()
+    m = 2 if mod == "qpsk" else 4
+    want = None
+    for chunk, kw in ((None, dict(PIPELINE=1)), (None, {}), (None, dict(PIPELINE=12)), (150_000, {}), (700_002, {})):
+        rx = make_receiver(p, LLR_OUT=form, BPS_HALFWIN=nb, **kw)
+        o = rx.run_stream(x, chunk=chunk, llr=True)
+        got = o["llr"][:, :o["n"] * m].clone()
+        rx.close()
+        want = got if want is None else want
+        assert torch.equal(got, want), (chunk, kw)
