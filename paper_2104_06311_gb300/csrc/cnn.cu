@@ -222,8 +222,10 @@ __global__ void __launch_bounds__(kThreads, 1) conv_kernel(const ConvArgs a) {
 // P[m][4 t + c] = sum_ci h[m][ci] W[t][ci][c] (4 MMAs per tile, N = 64), and
 // out[n][c] = sum_t P[n + t - 7][4 t + c] is 15 float4 additions per symbol.  A tile of
 // 128 rows gives 114 symbols.  Both edge kernels are bound by the 128-byte rows they
-// write or read and the latency of their phases; six and four CTAs share an SM: 39 and 47 us
-// at 2^20 symbols (mma.sync 182 and 269).
+// write or read and the latency of their phases; six (five with the mask of the layer below)
+// and four CTAs share an SM.  A network of the two alone takes 92 us at 2^20 symbols (mma.sync
+// 468; 114 where the 64 -> 4 kernel, with no residency stated, took 72 registers and spilled
+// 100 bytes).
 constexpr int TC_M = 128;                      // rows per tile (one MMA M)
 constexpr int TC_ROWS = TC_M + 2 * HALF;       // 142 rows per TMA box
 constexpr int TC_STAGES = 3;
@@ -245,6 +247,11 @@ constexpr long long kTcWaitNs = 2000000000ll;  // bounded waits
 constexpr int ED_W_BYTES = KS * CH * 16;       // weights of a 4 -> 64 layer: 16 bytes per tap and output
 constexpr int ED_TILE = TC_M - 2 * HALF;       // 114 symbols per tile of the 64 -> 4 layer
 constexpr unsigned ED_TMEM_COLS = 64;
+// CTAs of an edge kernel that one SM holds, by shared memory (37 and 57 KB) and registers (64, 96
+// and 100 of each thread): the persistent grids are one wave of them, a CTA more per SM would
+// start when the others end and load the weights again.  (The occupancy calculator answers 1
+// for kernels with tensor memory.)
+constexpr int ED_IN_CTAS = 6, ED_DX_CTAS = 5, ED_OUT_CTAS = 4;
 
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits
 // 7-9 = 1, 10-12 = 1), both K-major (bits 15, 16 = 0), N >> 3 at bits 17-22,
@@ -633,7 +640,7 @@ __global__ void __launch_bounds__(TC_M) edge_in_kernel(const __grid_constant__ C
 // 64 -> 4 with the residual output and, in training, dJ/dy and the loss (EPI_LAST).
 constexpr int ED_OUT_A = 0, ED_OUT_W = TC_OUT_BYTES, ED_OUT_P = ED_OUT_W + CH * CH * 2;
 constexpr int ED_OUT_SMEM = ED_OUT_P + KS * TC_M * 16 + 1024;   // + slack to align the base
-__global__ void __launch_bounds__(TC_M) edge_out_kernel(const __grid_constant__ CUtensorMap tin, const ConvArgs a,
+__global__ void __launch_bounds__(TC_M, ED_OUT_CTAS) edge_out_kernel(const __grid_constant__ CUtensorMap tin, const ConvArgs a,
                                                         const void *__restrict__ wimg, int *__restrict__ err) {
   extern __shared__ unsigned char tc_raw[];
   unsigned char *const sm = tc_raw + ((1024u - (smem_u32(tc_raw) & 1023u)) & 1023u);
@@ -1400,7 +1407,7 @@ cudaError_t launch_edge_in(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool p
   CUtensorMap tout;
   const cudaError_t e = row_map(&tout, a.out, a.K, 32);
   if (e != cudaSuccess) return e;
-  return launch_tc(edge_in_kernel<SRC_Z, EPI>, tc_grid(c, a.K, TC_M, 6), TC_M, 0, c->stream, pdl, tout, a,
+  return launch_tc(edge_in_kernel<SRC_Z, EPI>, tc_grid(c, a.K, TC_M, EPI == EPI_MASK ? ED_DX_CTAS : ED_IN_CTAS), TC_M, 0, c->stream, pdl, tout, a,
                    (const void *)img, c->err);
 }
 
@@ -1409,7 +1416,7 @@ cudaError_t launch_edge_out(rx_cnn *c, const ConvArgs &a, const bf16 *img, bool 
   CUtensorMap tin;
   const cudaError_t e = row_map(&tin, a.in, a.K, TC_M);
   if (e != cudaSuccess) return e;
-  return launch_tc(edge_out_kernel, tc_grid(c, a.K, ED_TILE, 4), TC_M, ED_OUT_SMEM, c->stream, pdl, tin, a,
+  return launch_tc(edge_out_kernel, tc_grid(c, a.K, ED_TILE, ED_OUT_CTAS), TC_M, ED_OUT_SMEM, c->stream, pdl, tin, a,
                    (const void *)img, c->err);
 }
 
