@@ -1251,6 +1251,7 @@ struct rx_cnn {
   int *err = nullptr;                  // sticky device error word (bounded waits), in res
   bf16 *x0 = nullptr, *dout = nullptr;
   std::vector<bf16 *> dz;              // dJ/d(pre-activation) of layers 0 .. L-2
+  bool dz_shared = false;              // ... two buffers in turn (the device had no room for all)
   std::vector<bf16 *> h;               // hidden outputs h_1 .. h_{L-1}
   struct Result { double loss; int err, pad; };
   Result *res = nullptr, *h_res = nullptr;   // device, and the pinned copy that grads reads back
@@ -1442,8 +1443,10 @@ cudaError_t launch_dw(rx_cnn *c, const bf16 *in, const bf16 *dz, int64_t K, int 
   return cudaGetLastError();
 }
 
-// Every layer's gradients into G (zeroed before the forward pass) from the stored rows.
-cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, float *G) {
+// Gradients of the layers [l0, l1) into G (zeroed before the forward pass) from the stored rows.
+// A launch of all of them comes behind the input gradients and may overlap the last of those; one of
+// a single layer may follow the kernel that wrote dJ/dy, which it reads through __ldg.
+cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, float *G, int l0, int l1) {
   KTimer tm(c, RX_CNN_K_DW);
   DwTcArgs a;
   memset(&a, 0, sizeof(a));
@@ -1452,7 +1455,8 @@ cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, floa
   const int64_t n_tiles = (K + TC_M - 1) / TC_M;
   // one wave of at most three CTAs per SM: two per SM over the hidden layers, a half over each
   // edge layer
-  const int64_t want_h = std::max<int64_t>(1, 2 * c->sms / (DW_GROUPS * std::max(1, c->L - 2)));
+  const int hidden = std::min(l1, c->L - 1) - std::max(l0, 1);
+  const int64_t want_h = std::max<int64_t>(1, 2 * c->sms / (DW_GROUPS * std::max(1, hidden)));
   const int64_t want_e = std::max(1, c->sms / 2);
   int blocks = 0;
   for (int l = 0; l < c->L; ++l) {
@@ -1460,7 +1464,8 @@ cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, floa
     const bool edge = l == 0 || l == c->L - 1;
     const int64_t chunk = (n_tiles + (edge ? want_e : want_h) - 1) / (edge ? want_e : want_h);
     y.chunk_tiles = (int)chunk;
-    y.first_block = blocks;
+    y.first_block = blocks;                            // (a layer outside the range has no blocks)
+    if (l < l0 || l >= l1) continue;
     blocks += (int)((n_tiles + chunk - 1) / chunk) * (edge ? 1 : DW_GROUPS);
     y.dw = G + c->off_w[l];
     y.db = G + c->off_b[l];
@@ -1471,7 +1476,7 @@ cudaError_t launch_dw_tc(rx_cnn *c, const float2 *z, int64_t zs, int64_t K, floa
     if (e == cudaSuccess && !edge) e = row_map(&y.x, c->h[l - 1], K, TC_ROWS);
     if (e != cudaSuccess) return e;
   }
-  return launch_tc(dw_tc_kernel, blocks, TC_M, DW_SMEM, c->stream, true, a, c->err);
+  return launch_tc(dw_tc_kernel, blocks, TC_M, DW_SMEM, c->stream, l1 - l0 == c->L, a, c->err);
 }
 
 rx_status check_sym(rx_cnn *c, const float *p, int64_t stride, int64_t K, const char *what) {
@@ -1543,6 +1548,8 @@ rx_status backward(rx_cnn *c, const float *z, int64_t zs, int64_t K, float *G) {
   for (int l = L - 1; l >= 0; --l) {
     const bool last = l == L - 1;
     const bf16 *dz = last ? c->dout : c->dz[l];      // [K][16] for the last layer
+    if (c->use_tc && c->dz_shared)
+      CX_CUDA(launch_dw_tc(c, reinterpret_cast<const float2 *>(z), zs, K, G, l, l + 1), "weight gradient");
     if (!c->use_tc) {
       if (l == 0) {
         CX_CUDA((launch_dw<FEATP, CH>(c, c->x0, dz, K, l, G)), "weight gradient");
@@ -1571,7 +1578,8 @@ rx_status backward(rx_cnn *c, const float *z, int64_t zs, int64_t K, float *G) {
       CX_CUDA((launch_conv<CH, CH, EPI_MASK>(c, a)), "input gradient");
     }
   }
-  if (c->use_tc) CX_CUDA(launch_dw_tc(c, reinterpret_cast<const float2 *>(z), zs, K, G), "weight gradients");
+  if (c->use_tc && !c->dz_shared)
+    CX_CUDA(launch_dw_tc(c, reinterpret_cast<const float2 *>(z), zs, K, G, 0, L), "weight gradients");
   return RX_OK;
 }
 
@@ -1653,7 +1661,7 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
   CX_ALLOC(c->x0, K * FEATP);
   CX_ALLOC(c->dout, K * FEATP);
   c->dz.assign(layers - 1, nullptr);
-  for (int l = 0; l < layers - 1; ++l) CX_ALLOC(c->dz[l], K * CH);
+  for (int l = 0; l < std::min(2, layers - 1); ++l) CX_ALLOC(c->dz[l], K * CH);
   c->h.assign(layers - 1, nullptr);
   for (int l = 0; l < layers - 1; ++l) CX_ALLOC(c->h[l], K * CH);
   CX_ALLOC(c->res, 1);
@@ -1665,6 +1673,15 @@ rx_status rx_cnn_create(rx_cnn **out, int layers, int channels, int ksize, int64
     return cfail(c, RX_ENOMEM, "pinned result");
   }
 #undef CX_ALLOC
+  // a buffer per layer lets one launch form every weight gradient from them; without room for
+  // that, two serve the layers in turn and each layer's gradient is formed before its turn ends
+  const size_t kept = c->allocs.size();
+  for (int l = 2; l < layers - 1 && !c->dz_shared; ++l) c->dz_shared = calloc_dev(c, &c->dz[l], K * CH) != RX_OK;
+  if (c->dz_shared) {
+    for (; c->allocs.size() > kept; c->allocs.pop_back()) cudaFree(c->allocs.back());
+    for (int l = 2; l < layers - 1; ++l) c->dz[l] = c->dz[l & 1];
+    c->msg.clear();
+  }
   CX_CUDA(cudaMemset(c->P, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->M, 0, (size_t)c->n_params * sizeof(float)), "init");
   CX_CUDA(cudaMemset(c->V, 0, (size_t)c->n_params * sizeof(float)), "init");

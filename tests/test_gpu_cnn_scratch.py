@@ -1,0 +1,52 @@
+"""The learned post-equaliser where the device has room for two gradient buffers but not for
+one per layer: the handle is created all the same and its gradients are those of a handle with
+all of them (the same BF16 values; the FP32 sums differ in the order of their atomics)."""
+import pytest
+
+from chain_helpers import ensure_built, rel_rms
+from test_gpu_cnn import _data, _dev
+from test_gpu_cnn_edges import _net
+
+pytestmark = pytest.mark.gpu
+
+LAYERS, K_MAX = 8, 1 << 20
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    ensure_built()
+
+
+@pytest.mark.parametrize("K", [131, 5000])
+def test_two_gradient_buffers(K):
+    import torch
+    z, t = _data(K, 41)
+    z, t = _dev(z), _dev(t)
+    roomy = _net(K_MAX, LAYERS)
+    want = {}
+    for tc in (1, 0):
+        roomy.set_option("TCGEN05", tc)
+        loss, g = roomy.grads(z, t)
+        want[tc] = loss, roomy.unflatten(g.cpu().numpy())
+    roomy.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    # rows of 128 bytes: 7 activations, 2 gradients, 32 bytes twice; a handle with 5 more does not fit
+    need = K_MAX * (9 * 128 + 64)
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - need - (256 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        left, _ = torch.cuda.mem_get_info()
+        assert need < left < need + K_MAX * 4 * 128
+        net = _net(K_MAX, LAYERS)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    for tc in (1, 0):
+        net.set_option("TCGEN05", tc)
+        loss, g = net.grads(z, t)
+        g = net.unflatten(g.cpu().numpy())
+        assert abs(loss - want[tc][0]) < 1e-9 * want[tc][0]
+        for (dW, db), (rW, rb) in zip(g, want[tc][1]):
+            assert rel_rms(dW, rW) < 1e-5 and rel_rms(db, rb) < 1e-5
+    net.close()
