@@ -215,7 +215,8 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
     // exp(j (phi + 2 pi f_c s / fs)): the turn s inc_q (signed Q0.64) in half turns to 32
     // bits, phi / pi in two terms, one sine and cosine
     const float turn = (float)(int)(((unsigned long long)s * inc_q) >> 32) * 4.65661287307739258e-10f;   // 2^-31
-    const float phi = ph[m];
+    // (a 0 there whatever the phase: an infinite intensity leaves none in its whole window)
+    const float phi = a > 0.f ? ph[m] : 0.f;
     float sp, cp;
     sincospif(fmaf(phi, 0.31830987334251404f, fmaf(phi, 1.2841276632e-08f, turn)), &sp, &cp);
     E[s - e0] = make_float2(a * cp, a * sp);

@@ -25,3 +25,16 @@ def test_short_buffers(adc, bufs):
     yg, fg = _stream(fe, g.samples, cuts, g)
     yo, Eo, _ = K.kk_frontend(g.samples, g.in_scale, g.in_offset, lk.baud, lk.sps, lk.carrier_hz, lk.L_km)
     assert rel_rms(fg, Eo) < TOL and rel_rms(yg, yo) < TOL
+
+
+@pytest.mark.parametrize("at", [0, 100, 255])
+def test_field_outside_the_stream_is_zero(at):
+    # an infinite intensity takes the phase of its window from the samples around it; in front of the
+    # stream there is no field all the same
+    import torch
+    from paper_2104_06311_gb300 import KKFrontEnd
+    fe = KKFrontEnd(1e9, 0.516e9, 1000.0, 4096)
+    x = torch.ones(4096, device="cuda")
+    x[at] = float("inf")
+    _, field = fe.process(x, field=True)
+    assert torch.all(field[:fe.delay] == 0)
