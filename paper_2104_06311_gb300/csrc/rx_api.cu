@@ -815,7 +815,6 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       // two counter sets in turn: each launch zeroes the other one for the next
       L.barrier = rx->barrier + (rx->bar_set ? kEqBarrierWords : 0);
       L.barrier_next = rx->barrier + (rx->bar_set ? 0 : kEqBarrierWords);
-      rx->bar_set = !rx->bar_set;
       L.err = rx->err;
       L.K = K;
       L.run_acq = j == 0 && run_acq;
@@ -849,6 +848,7 @@ rx_status rx_process(rx_stream *rx, const rx_in *in, rx_out *out) {
       StageTimer tm(rx, RX_STAGE_EQ, rx->sub[1]);
       rx->stage_launches[RX_STAGE_EQ] += 1;
       RX_CUDA(launch_eq(L, rx->sub[1]), "equaliser");
+      rx->bar_set = !rx->bar_set;   // (a launch that failed has zeroed nothing)
       wa = wb;
     }
     RX_CUDA(cudaEventRecord(rx->ev_piece[1][j], rx->sub[1]), "event");
