@@ -1,6 +1,8 @@
-"""The learned post-equaliser where the device has room for two gradient buffers but not for
-one per layer: the handle is created all the same and its gradients are those of a handle with
-all of them (the same BF16 values; the FP32 sums differ in the order of their atomics)."""
+"""Buffers of the learned post-equaliser.  Where the device has room for two gradient buffers
+but not for one per layer, the handle is created all the same and its gradients are those of a
+handle with all of them (the same BF16 values; the FP32 sums differ in the order of their
+atomics).  A caller's gradient buffer that is not on a 16-byte boundary is filled like any
+other, and nothing beside it is written."""
 import pytest
 
 from chain_helpers import ensure_built, rel_rms
@@ -49,4 +51,26 @@ def test_two_gradient_buffers(K):
         assert abs(loss - want[tc][0]) < 1e-9 * want[tc][0]
         for (dW, db), (rW, rb) in zip(g, want[tc][1]):
             assert rel_rms(dW, rW) < 1e-5 and rel_rms(db, rb) < 1e-5
+    net.close()
+
+
+@pytest.mark.parametrize("layers,offset", [(2, 1), (4, 1), (4, 2), (4, 3)])
+def test_gradient_buffer_off_the_16_byte_boundary(layers, offset):
+    import ctypes as ct
+    import torch
+    z, t = _data(777, 43)
+    z, t = _dev(z), _dev(t)
+    net = _net(1000, layers)
+    want_loss, want = net.grads(z, t)
+    buf = torch.full((net.n_params + 8,), 7.5, device="cuda")
+    assert buf.data_ptr() % 16 == 0
+    loss = ct.c_double()
+    torch.cuda.synchronize()
+    st = net.lib.rx_cnn_grads(net.h, z.data_ptr(), z.stride(0), t.data_ptr(), t.stride(0), 777,
+                              buf.data_ptr() + 4 * offset, ct.byref(loss))
+    assert st == 0 and abs(loss.value - want_loss) < 1e-9 * want_loss
+    g, w = net.unflatten(buf[offset:offset + net.n_params].cpu().numpy()), net.unflatten(want.cpu().numpy())
+    for (dW, db), (rW, rb) in zip(g, w):           # (FP32 atomics in another order)
+        assert rel_rms(dW, rW) < 1e-5 and rel_rms(db, rb) < 1e-5
+    assert torch.all(buf[:offset] == 7.5) and torch.all(buf[offset + net.n_params:] == 7.5)
     net.close()

@@ -38,3 +38,25 @@ def test_field_outside_the_stream_is_zero(at):
     x[at] = float("inf")
     _, field = fe.process(x, field=True)
     assert torch.all(field[:fe.delay] == 0)
+
+
+@pytest.mark.parametrize("carrier", [0.516321e9, 1.2345e9, 1.9990001e9])
+@pytest.mark.parametrize("pos", [0, 512 * 123457])
+def test_carrier_phase_off_the_recording_grid(carrier, pos):
+    # intensity 1 everywhere: amplitude 1, phase 0, so the field is the carrier's turn alone.  Its
+    # error: 24 significant bits of the half turn (pi 2^-25), one unit in the last place of the
+    # sine and of the cosine (2^-24 each near 1) and of the product with the amplitude
+    import math
+    import numpy as np
+    import torch
+    from paper_2104_06311_gb300 import KKFrontEnd
+    n = 8192
+    fe = KKFrontEnd(1e9, carrier, 1000.0, n)
+    fe.set_position(pos)
+    _, field = fe.process(torch.ones(n, device="cuda"), field=True)
+    f = field.cpu().numpy().astype(np.complex128)[fe.delay:]
+    inc = int(carrier / 4e9 % 1.0 * 2.0 ** 64)                 # exact: a double's 53 bits
+    turn = np.array([((pos + i) * inc % (1 << 64)) / 2.0 ** 64 for i in range(f.shape[0])])
+    err = np.abs(f - np.exp(2j * np.pi * turn))
+    print(f"carrier {carrier:.6g} from {pos}: max {err.max():.2e}")
+    assert err.max() < math.pi * 2.0 ** -25 + math.sqrt(2) * 2 * 2.0 ** -24
