@@ -74,3 +74,38 @@ def test_gradient_buffer_off_the_16_byte_boundary(layers, offset):
         assert rel_rms(dW, rW) < 1e-5 and rel_rms(db, rb) < 1e-5
     assert torch.all(buf[:offset] == 7.5) and torch.all(buf[offset + net.n_params:] == 7.5)
     net.close()
+
+
+def test_first_use_by_several_threads():
+    # every convolution needs the driver's tensor-map entry point, looked up at the first use: in a
+    # process of its own, so that this is the first
+    import subprocess
+    import sys
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = """
+import sys, threading
+sys.path[:0] = [%r, %r]
+import torch
+from test_gpu_cnn import _data, _dev
+from test_gpu_cnn_edges import _net
+z = _dev(_data(5000, 47)[0])
+n = 8
+nets = [_net(5000, 4) for _ in range(n)]
+torch.cuda.synchronize()
+gate, out, bad = threading.Barrier(n), [None] * n, []
+def work(i):
+    try:
+        gate.wait()
+        out[i] = nets[i].apply(z)
+    except Exception as e:
+        bad.append(repr(e))
+ts = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+[t.start() for t in ts]
+[t.join() for t in ts]
+torch.cuda.synchronize()
+assert not bad, bad
+assert all(torch.equal(o, out[0]) for o in out)
+""" % (root, os.path.join(root, "tests"))
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr[-2000:]
