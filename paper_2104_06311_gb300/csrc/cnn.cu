@@ -1362,11 +1362,20 @@ cudaError_t row_map(CUtensorMap *m, const bf16 *p, int64_t K, unsigned rows) {
   const cuuint64_t strides[1] = {(cuuint64_t)CH * sizeof(bf16)};
   const cuuint32_t box[2] = {(cuuint32_t)CH, rows};
   const cuuint32_t estr[2] = {1u, 1u};
-  if (enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(p), dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-    return cudaErrorInvalidValue;
-  return cudaSuccess;
+  auto encode = [&]() {
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16 *>(p), dims, strides, box, estr,
+               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  };
+  CUresult r = encode();
+  if (r == CUDA_ERROR_INVALID_CONTEXT || r == CUDA_ERROR_NOT_INITIALIZED) {
+    // a host thread whose first CUDA call this is: the driver, unlike the runtime, does not bind
+    // the device's context by itself
+    const cudaError_t e = cudaFree(nullptr);
+    if (e != cudaSuccess) return e;
+    r = encode();
+  }
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 // A launch that may start its prologue while the kernel in front of it drains (pdl).

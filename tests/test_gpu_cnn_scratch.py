@@ -77,8 +77,8 @@ def test_gradient_buffer_off_the_16_byte_boundary(layers, offset):
 
 
 def test_first_use_by_several_threads():
-    # every convolution needs the driver's tensor-map entry point, looked up at the first use: in a
-    # process of its own, so that this is the first
+    # every convolution needs the driver's tensor-map entry point, looked up at the first use, and a
+    # context, which a new thread has not bound: in a process of its own, so that this is the first
     import subprocess
     import sys
     import os
