@@ -79,10 +79,11 @@ enum {
 
 /* Options for rx_cnn_set_option. */
 enum {
-  RX_CNN_OPT_TCGEN05 = 1    /* 1 (default): the 64 -> 64 convolutions (forward and
-                               input gradient) run on tcgen05 / tensor memory;
-                               0: on warp-level mma.sync (BF16, FP32 accumulate),
-                               the kernel the first and last layers always use   */
+  RX_CNN_OPT_TCGEN05 = 1    /* 1 (default): every convolution (forward and input
+                               gradient, the 4 -> 64 and 64 -> 4 layers among them)
+                               and every weight gradient run on tcgen05 / tensor
+                               memory; 0: all of them on warp-level mma.sync.
+                               BF16 in, FP32 accumulate either way                */
 };
 rx_status rx_cnn_set_option(rx_cnn *c, int key, int value);
 

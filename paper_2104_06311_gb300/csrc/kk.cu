@@ -212,8 +212,9 @@ __global__ void __launch_bounds__(KT, 12) kk_hilbert_kernel(KkSrc src, int64_t e
     const int m = t + KT * i;                    // field sample of the pair
     const int64_t s = lo + KH / 2 + m;
     const float a = amp[m];                      // outside the stream: zero field
-    // exp(j (phi + 2 pi f_c s / fs)): the turn s inc_q (signed Q0.64) in half turns to 32
-    // bits, phi / pi in two terms, one sine and cosine
+    // exp(j (phi + 2 pi f_c s / fs)): the turn s inc_q (signed Q0.64) in half turns, rounded from
+    // its top 32 bits to the 24 of a float (2^-25 half turns near +-1), phi / pi in two terms,
+    // one sine and cosine
     const float turn = (float)(int)(((unsigned long long)s * inc_q) >> 32) * 4.65661287307739258e-10f;   // 2^-31
     // (a 0 there whatever the phase: an infinite intensity leaves none in its whole window)
     const float phi = a > 0.f ? ph[m] : 0.f;

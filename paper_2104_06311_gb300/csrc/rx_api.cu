@@ -335,15 +335,15 @@ unsigned char *u_at(rx_stream *rx, int b, int p, int64_t n) {
   return reinterpret_cast<unsigned char *>(rx->u[b]) + (p * rx->u_cap + n) * fmt_bytes(rx->fmt);
 }
 
-// Region layout: region 0 = [0, A), region r >= 1 = [A + (r-1) span, A + r span).
 // Pieces of a call of n waves when the caller names none.  A piece hides what comes before
 // and after it (the first piece's CDC and the last one's BPS stay in the open: about
 // 4 us per wave of the piece) and costs the equaliser's start and drain, 13 to 16 us of a
 // launch: the sum is least near sqrt(n) / 2 pieces, and pieces also wait on their CDC
-// beside the equaliser, so the line lies a little below (10 GBd QPSK, 512 waves: 3, 5, 6, 8,
-// 10 pieces 9.89, 9.48, 9.43, 9.38, 9.32 ms; 32 GBd 16QAM, 31 waves: 1, 2, 4, 12 pieces
-// 1082, 1033, 1040, 1190 us; 21 waves: 1, 2, 4, 12 pieces 802, 775, 796, 930 us; calls of 9
-// waves: 1, 2, 12 pieces 1636, 1789, 2043 us).
+// beside the equaliser, so the line lies a little below.  Measured: 10 GBd QPSK, 512 waves
+// (9 pieces by the rule): 3, 5, 6, 8, 9, 10, 12 pieces 9.26, 9.48, 9.40, 9.42, 9.31, 9.29,
+// 9.24 ms; 32 GBd 16QAM, 31 waves (2): 1, 2, 3, 4, 12 pieces 1058, 1004, 978, 1016, 1134 us;
+// 21 waves (2): 1, 2, 3, 4, 12 pieces 768, 762, 751, 778, 856 us; a stream of nine calls of
+// four to five waves each (1): 1, 2, 3, 12 pieces 1495, 1628, 1637, 1856 us.
 int auto_pieces(const rx_stream *rx, int64_t n) {
   return (int)std::min<double>(rx->pieces, std::max(1.0, floor(0.4 * sqrt((double)n) + 0.5)));
 }
@@ -359,6 +359,7 @@ int bps_chunk(const rx_stream *rx, int64_t n) {
   return c;
 }
 
+// Region layout: region 0 = [0, A), region r >= 1 = [A + (r-1) span, A + r span).
 int64_t region_end_after(const rx_stream *rx, int64_t k) {
   // end of the region that starts at or contains symbol k
   if (k < rx->A) return rx->A;

@@ -261,18 +261,6 @@ __global__ void __launch_bounds__(WBLOCK) wl_kernel(const float4 *__restrict__ x
   }
 }
 
-// Widely-linear form on four lanes per segment (8 segments per warp).  With M_i as above,
-// Re z and Im z are two recursions that share only their input: Re e updates the upper
-// rows (m00, m01) and Im e the lower ones.  Lane 2 comp + half runs component comp over
-// the taps i = half, half + 2: its half of the dot product M u and of the look-ahead's
-// u(k-1) . u(k), one exchange each with the other half, the decision, and the update of its
-// own four entries.  Every sum is formed in the order of a plain one-lane form.  What counts
-// is a warp's instructions per symbol and what waits: the next symbol's half sums and their
-// exchange stand in front of this symbol's decision, which takes as long.  Per symbol: one
-// lane 68 ns (561 us for the acquisition's 8192), four lanes with the exchange behind the
-// decision 46, two lanes (no exchange, twice the sums) 43, this form 37.
-// The segments of a warp run in lockstep over [s0 - W, s0 + S); where one starts later or
-// ends earlier its state holds.
 // e' = mu_s (dec(z) - z) of one component, with wl_decide's level: its sign and size (16QAM)
 // as flags.  Both levels' errors are formed while |z| is compared: one select at the end
 // of the chain.
@@ -290,6 +278,18 @@ __device__ __forceinline__ float wl_error(float z, float mu_s, bool &neg, bool &
   return outer ? e3 : e1;
 }
 
+// Widely-linear form on four lanes per segment (8 segments per warp).  With M_i as above,
+// Re z and Im z are two recursions that share only their input: Re e updates the upper
+// rows (m00, m01) and Im e the lower ones.  Lane 2 comp + half runs component comp over
+// the taps i = half, half + 2: its half of the dot product M u and of the look-ahead's
+// u(k-1) . u(k), one exchange each with the other half, the decision, and the update of its
+// own four entries.  Every sum is formed in the order of a plain one-lane form.  What counts
+// is a warp's instructions per symbol and what waits: the next symbol's half sums and their
+// exchange stand in front of this symbol's decision, which takes as long.  Per symbol: one
+// lane 68 ns (561 us for the acquisition's 8192), four lanes with the exchange behind the
+// decision 46, two lanes (no exchange, twice the sums) 43, this form 36.
+// The segments of a warp run in lockstep over [s0 - W, s0 + S); where one starts later or
+// ends earlier its state holds.
 template <int MB>
 struct WlRec4 {
   float a0, a1, b0, b1;      // this component's factors of Re, Im u: taps half (a) and half + 2 (b)
