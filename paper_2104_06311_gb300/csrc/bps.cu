@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_slide(BpsLaunch L) {
   // window of symbol `start`.  The re-sum below adds the ring by slots, so the order of a sum
   // is that of a chunk begun at the last grid point, whatever the length of this one: a near
   // tie falls the same way however a recording is cut into calls, pieces and chunks
-  const int o = (int)((a - L.k_lo) % L.grid) % M;
+  const int o = (int)((a - L.k_lo) & (L.grid - 1)) % M;
   for (int i = 0; i < M; ++i) {
     const int q = o + i;
     ring[(q < M ? q : q - M) * 32 + lane] = dist(i);

@@ -118,8 +118,9 @@ struct BpsLaunch {
   int64_t K_end;            // symbols known to exist (stream end if flushed)
   int64_t A, span;          // region layout
   int chunk;                // chunk length (symbols)
-  int grid;                 // a multiple of chunk that regions start on: the sliding pass adds its
-                            // window in an order that depends on the position on this grid alone
+  int grid;                 // a multiple of chunk and a power of two that regions start on: the
+                            // sliding pass adds its window in an order that depends on the
+                            // position on this grid alone
   int part;                 // 32 or 64, divides chunk: symbols of an FP32 partial sum of the noise
                             // variance, the same for every chunk length, so that an LLR does not
                             // depend on how the recording is cut
