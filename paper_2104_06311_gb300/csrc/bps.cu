@@ -339,9 +339,9 @@ __global__ void __launch_bounds__(kBpsWarps * 32) bps_pass1_blk(BpsLaunch L) {
 // one thread each took 17.5 us of a call's tail at 128 sums per region, the warps take 10 at
 // 512.  Without LLRs (NEED_S2 false) it keeps to 32 registers, some words spilled: with more a
 // CTA waits longer for room beside the other kernels of a batch (64 channels, 56 registers:
-// 6166 -> 6194 us).  The
-// regions take up to 64: 2^20 16QAM symbols with LLRs 993 us either way, 700,001 with FP16 LLRs
-// 745 us at 32 and a few words spilled, 743 at 64, six channels 389 and 387.
+// 6166 -> 6194 us; 32 without the spills, chunk loops not unrolled: no change).  The regions
+// take up to 64: 2^20 16QAM symbols with LLRs 993 us either way, 700,001 with FP16 LLRs 745 us
+// at 32 and a few words spilled, 743 at 64, six channels 389 and 387.
 template <bool NEED_S2>
 __global__ void __launch_bounds__(1024, NEED_S2 ? 1 : 2) bps_scan(BpsLaunch L) {
   __shared__ int64_t part[32];
